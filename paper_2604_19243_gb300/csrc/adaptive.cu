@@ -483,7 +483,7 @@ fmm_status afail(fmm_ctx *ctx, fmm_status st, const std::string &m) {
     return st;
 }
 
-constexpr int kAdaptTile = 64;   // rows per tile of the far pass's GEMMs (the SIMT form's)
+constexpr int kAdaptTile = 128;   // rows per tile of the far pass's GEMMs
 
 template <typename V>
 cudaError_t upload_vec(const std::vector<V> &h, V **d) {
@@ -855,6 +855,27 @@ fmm_status adaptive_prepare(fmm_ctx *ctx) {
     return FMM_OK;
 }
 
+// VLI stencil of one level over its kept boxes: FP64 by the SIMT GEMM, FP32 from three FP16 planes
+// on the tensor cores (gemm_f16.cu), in the uniform tree's groups of transfer vectors.
+template <typename T>
+static cudaError_t adaptive_stencil(fmm_ctx *ctx, GemmCall st, const AdaptiveLevel &L, cudaStream_t s) {
+    if (!ctx->f32m2l) return gemm_simt<T>(ctx, st, s);
+    const int l = st.level, kw = ctx->ws_kw;
+    const OpSet &o = ctx->fwd[l];
+    const size_t rb = (size_t)ctx->lev[l].row_base;
+    st.Xp = (unsigned char *)ctx->UtP + rb * kw * 2, st.xp_ld = kw, st.xp_plane = ctx->utp_plane;
+    st.xp_scale = ctx->Uscale + rb;
+    FMM_CUDA_TRY(launch_rows_planes((const float *)st.X0, 0, 1, kw, L.kept, L.n_kept, o.kinp, nullptr, 0, (void *)st.Xp,
+                                    ctx->utp_plane, kw, ctx->Uscale + rb, 1, 3, s));
+    float *ct = (float *)st.Y;
+    st.groups = stencil_groups(o, l);
+    if (st.groups > 1) st.Y = ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
+    FMM_CUDA_TRY(gemm_f16(ctx, st, o.f_stencil, nullptr, s));
+    if (st.groups == 1) return cudaSuccess;
+    return launch_rows_planes((const float *)st.Y, st.y_group, st.groups, kw, L.kept, L.n_kept, o.koutp, ct, kw, nullptr,
+                              0, kw, nullptr, 1, 3, s);
+}
+
 // The far field over the adaptive tree (forward, FP32/FP64): far_phi / far_grad (sorted order)
 // receive D2T and WLI of every point.
 template <typename T>
@@ -905,7 +926,7 @@ cudaError_t adaptive_far(fmm_ctx *ctx, T *far_phi, T *far_grad, cudaStream_t s) 
             st.Y = at(ctx->Ct, l, kw), st.ldy = kw;
             st.dense = A->dense_kept[l];
             restrict_to(st, L.kept_tiles, L.kept);
-            FMM_CUDA_TRY(gemm_simt<T>(ctx, st, ls));
+            FMM_CUDA_TRY(adaptive_stencil<T>(ctx, st, L, ls));
         }
         FMM_CUDA_TRY(cudaEventRecord(ctx->join_ev[l], ls));
     }

@@ -116,6 +116,7 @@ void free_workspace(fmm_ctx *ctx) {
     if (ctx->masks_ev) cudaStreamWaitEvent(s, ctx->masks_ev, 0);   // the side stream's mask kernels
     free_async(ctx->Uc, s), free_async(ctx->Dc, s), free_async(ctx->Ut, s), free_async(ctx->Ct, s);
     free_async(ctx->UtP, s), free_async(ctx->Uscale, s);
+    free_async(ctx->StP, s);
     free_async(ctx->UpP, s), free_async(ctx->DnP, s), free_async(ctx->CtP, s);
     free_async(ctx->Ups, s), free_async(ctx->Dns, s), free_async(ctx->Cts, s);
     free_async(ctx->Yc, s), free_async(ctx->Dq, s), free_async(ctx->Cmean, s);
@@ -171,11 +172,21 @@ void free_ops(fmm_ctx *ctx) {
 // passes); the tiles of the VLI and the level sweeps are rebuilt for every tree.
 fmm_status ensure_workspace(fmm_ctx *ctx) {
     const int64_t need_rows = ctx->total_rows, need_nl = ctx->nleaf, need_n = ctx->n;
-    if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n))
+    // partial rows of the stencil's groups (gemm_f16.cu)
+    size_t stp = 0;
+    if (ctx->f16 || ctx->f32m2l) {
+        const OpSet &o = ctx->fwd[ctx->opt.depth];
+        const int kw = std::max(std::max(o.kinp, o.koutp), 16);
+        for (int l = 2; l <= ctx->opt.depth; ++l) {
+            ctx->stp_base[l] = (long long)stp;
+            if (stencil_groups(o, l) > 1) stp += (size_t)stencil_groups(o, l) * ctx->lev[l].n * kw;
+        }
+    }
+    if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n || stp > ctx->stp_floats))
         free_workspace(ctx);
     if (ctx->have_ws) {
         if (!ctx->tiles_ok) {
-            cudaError_t e = build_tiles(ctx, ctx->tensor ? 128 : 64);
+            cudaError_t e = build_tiles(ctx, ctx->fp64 ? 64 : 128);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "tile construction");
             ctx->tiles_ok = true;
         }
@@ -189,13 +200,15 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
     ctx->ws_kw = kw;
     const int64_t rows = need_rows, nl = need_nl, n = need_n;
     const int vc = ctx->cplx ? 2 : 1;   // values per point (complex outputs)
+    // FP32 rows of the compressed vectors: the SIMT modes, and FP16X3 when no CTA holds a whole row
+    const size_t ut_bytes = !ctx->tensor || (ctx->f16 && o.wide) ? (size_t)rows * kw * es : (size_t)16;
     struct A {
         void **p;
         size_t bytes;
     } allocs[] = {
         {&ctx->Uc, (size_t)rows * nsp * es},   {&ctx->Dc, (size_t)rows * nsp * es},
         // tensor-core modes hand the compressed vectors over as split planes (UtP) instead
-        {&ctx->Ut, ctx->tensor ? (size_t)16 : (size_t)rows * kw * es},
+        {&ctx->Ut, ut_bytes},
         {&ctx->Ct, (size_t)rows * kw * es},
         {&ctx->Yc, (size_t)nl * o.rclp * es},
         {&ctx->Dq, (size_t)nl * nsp * es},     {&ctx->Cmean, (size_t)rows * sizeof(double)},
@@ -203,35 +216,34 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         {&ctx->near_grad, (size_t)n * 3 * vc * es}, {&ctx->far_phi, (size_t)n * vc * es},
         {&ctx->far_grad, (size_t)n * 3 * vc * es}, {&ctx->pts_qi, ctx->cplx ? (size_t)n * es : (size_t)16},
     };
-    if (ctx->tensor) {
-        const int np = ctx->opt.precision == FMM_BF16X6 ? 3 : 2;
+    if (ctx->tensor || ctx->f32m2l) {
+        const int np = ctx->opt.precision == FMM_BF16X6 || ctx->f32m2l ? 3 : 2;
         const size_t pesz = ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
         ctx->utp_plane = (long long)((size_t)rows * kw * pesz + 256) / 256 * 256;
-        if (ctx->opt.precision == FMM_FP16X3) {
+        bool okp = pool_alloc(&ctx->UtP, (size_t)ctx->utp_plane * np, s) == cudaSuccess;
+        const size_t nsc = ctx->f16 && o.wide ? (size_t)(std::max(nsp, kw) + 63) / 64 : 1;   // scales a row
+        if (ctx->f16 || ctx->f32m2l)
+            okp = okp && pool_alloc((void **)&ctx->Uscale, (size_t)rows * nsc * sizeof(float) + 16, s) == cudaSuccess &&
+                  pool_alloc((void **)&ctx->StP, stp * sizeof(float) + 16, s) == cudaSuccess;
+        if (ctx->f16) {
             // every contraction reads FP16 planes: the upward- and downward-side rows, the
             // compressed vectors (UtP) and the stencil output, each with its row scales
             ctx->upp_plane = (long long)((size_t)rows * nsp * 2 + 256) / 256 * 256;
             ctx->ctp_plane = ctx->utp_plane;
-            const size_t ns_chunks = (size_t)rows * ((nsp + 63) / 64) * sizeof(float) + 16;
-            const size_t kw_chunks = (size_t)rows * ((kw + 63) / 64) * sizeof(float) + 16;
-            bool okp = pool_alloc((void **)&ctx->Uscale, kw_chunks, s) == cudaSuccess &&
-                       pool_alloc((void **)&ctx->Cts, kw_chunks, s) == cudaSuccess &&
-                       pool_alloc((void **)&ctx->Ups, ns_chunks, s) == cudaSuccess &&
-                       pool_alloc((void **)&ctx->Dns, ns_chunks, s) == cudaSuccess &&
-                       pool_alloc(&ctx->UpP, (size_t)ctx->upp_plane * 2, s) == cudaSuccess &&
-                       pool_alloc(&ctx->DnP, (size_t)ctx->upp_plane * 2, s) == cudaSuccess &&
-                       pool_alloc(&ctx->CtP, (size_t)ctx->ctp_plane * 2, s) == cudaSuccess;
-            if (!okp) {
-                cudaGetLastError();
-                free_workspace(ctx);
-                return fail(ctx, FMM_ENOMEM, "workspace allocation failed (FP16 planes)");
-            }
+            const size_t scales = (size_t)rows * nsc * sizeof(float) + 16;
+            okp = okp && pool_alloc((void **)&ctx->Cts, scales, s) == cudaSuccess &&
+                  pool_alloc((void **)&ctx->Ups, scales, s) == cudaSuccess &&
+                  pool_alloc((void **)&ctx->Dns, scales, s) == cudaSuccess &&
+                  pool_alloc(&ctx->UpP, (size_t)ctx->upp_plane * 2, s) == cudaSuccess &&
+                  pool_alloc(&ctx->DnP, (size_t)ctx->upp_plane * 2, s) == cudaSuccess &&
+                  pool_alloc(&ctx->CtP, (size_t)ctx->ctp_plane * 2, s) == cudaSuccess;
         }
-        if (pool_alloc(&ctx->UtP, (size_t)ctx->utp_plane * np, s) != cudaSuccess) {
+        if (!okp) {
             cudaGetLastError();
             free_workspace(ctx);
             return fail(ctx, FMM_ENOMEM, "workspace allocation failed (split planes)");
         }
+        ctx->stp_floats = stp;
     }
     size_t total = 0;
     for (auto &a : allocs) {
@@ -246,10 +258,10 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
     // rows that no step writes (levels 0-1, unused padding) must read as zero
     for (void **p : {&ctx->Uc, &ctx->Dc, &ctx->Ut, &ctx->Ct}) {
         size_t b = (p == &ctx->Uc || p == &ctx->Dc) ? (size_t)rows * nsp * es : (size_t)rows * kw * es;
-        if (p == &ctx->Ut && ctx->tensor) b = 16;
+        if (p == &ctx->Ut) b = std::max<size_t>(ut_bytes, 16);
         cudaMemsetAsync(*p, 0, b, s);
     }
-    cudaError_t e = build_tiles(ctx, ctx->tensor ? 128 : 64);
+    cudaError_t e = build_tiles(ctx, ctx->fp64 ? 64 : 128);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tile construction");
     ctx->tiles_ok = true;
     ctx->ws_bytes = total;
@@ -466,6 +478,8 @@ fmm_status fmm_create(const fmm_options *opt, void *cuda_stream, fmm_ctx **out) 
     ctx->fp64 = opt->precision == FMM_FP64;
     ctx->tensor = opt->precision == FMM_TF32X3 || opt->precision == FMM_BF16X3 || opt->precision == FMM_BF16X6 ||
                   opt->precision == FMM_FP16X3;
+    ctx->f16 = opt->precision == FMM_FP16X3;
+    ctx->f32m2l = opt->precision == FMM_FP32 && opt->m2l == FMM_M2L_DENSE;
     ctx->npts = 6 * (opt->order_p - 1) * (opt->order_p - 1) + 2;
     ctx->cplx = opt->kernel == FMM_HELMHOLTZ;
     ctx->fft = opt->m2l == FMM_M2L_FFT;

@@ -75,7 +75,16 @@ __global__ void remove_mean_kernel(T *__restrict__ D, int n, int ns, int ld, con
 template <typename T>
 cudaError_t gemm(const fmm_ctx *ctx, const GemmCall &c, int op_id, cudaStream_t s) {
     const int op = op_id % OP_COUNT;
-    if (ctx->tensor && op != OP_CLOSE1 && op != OP_CLOSE2) return gemm_tc(ctx, c, op_id, s);
+    if (op == OP_CLOSE1 || op == OP_CLOSE2) return gemm_simt<T>(ctx, c, s);
+    if (ctx->f16 || (ctx->f32m2l && op == OP_STENCIL)) {
+        const OpSet *set = op_id >= OP_COUNT ? ctx->adj : ctx->fwd;
+        const OpSet &o = set[c.level];
+        const F16Mat &w = op == OP_UP ? o.f_up : op == OP_COMPRESS ? o.f_compress
+                                              : op == OP_STENCIL  ? o.f_stencil
+                                                                  : o.f_decompress;
+        return gemm_f16(ctx, c, w, c.level > 0 ? &set[c.level - 1].f_down : nullptr, s);
+    }
+    if (ctx->tensor) return gemm_tc(ctx, c, op_id, s);
     return gemm_simt<T>(ctx, c, s);
 }
 
@@ -93,8 +102,7 @@ FarSteps<T>::FarSteps(fmm_ctx *c, bool adj) : ctx(c), adjoint(adj) {
     kw = ctx->ws_kw;
     A = adjoint ? ctx->Dc : ctx->Uc;
     B = adjoint ? ctx->Uc : ctx->Dc;
-    f16 = ctx->opt.precision == FMM_FP16X3;
-    nck_s = (nsp + 63) / 64, nck_k = (kw + 63) / 64;
+    f16 = ctx->f16;
 }
 
 // FMM_FP16X3: every contraction reads FP16 planes, which the step producing its input writes
@@ -109,12 +117,19 @@ template <typename T> unsigned char *FarSteps<T>::dnP(int l) const {
 template <typename T> unsigned char *FarSteps<T>::ctP(int l) const {
     return (unsigned char *)ctx->CtP + base(l) * kw * 2;
 }
-template <typename T> float *FarSteps<T>::upS(int l) const { return ctx->Ups + base(l) * nck_s; }
-template <typename T> float *FarSteps<T>::dnS(int l) const { return ctx->Dns + base(l) * nck_s; }
-template <typename T> float *FarSteps<T>::ctS(int l) const { return ctx->Cts + base(l) * nck_k; }
+template <typename T> float *FarSteps<T>::upS(int l) const { return ctx->Ups + base(l) * scales(nsp); }
+template <typename T> float *FarSteps<T>::dnS(int l) const { return ctx->Dns + base(l) * scales(nsp); }
+template <typename T> float *FarSteps<T>::ctS(int l) const { return ctx->Cts + base(l) * scales(O(d).koutp); }
 
 // operators of level l (one set for Laplace; per level for the modified Helmholtz kernel)
 template <typename T> const OpSet &FarSteps<T>::O(int l) const { return adjoint ? ctx->adj[l] : ctx->fwd[l]; }
+
+// FP32 rows of level l (n columns) to two planes
+template <typename T>
+cudaError_t FarSteps<T>::planes(const float *x, int n, int l, unsigned char *out, long long plane, float *inv_scale,
+                                cudaStream_t s) {
+    return launch_rows_planes(x, 0, 1, n, nullptr, ctx->lev[l].n, n, nullptr, 0, out, plane, n, inv_scale, scales(n), 2, s);
+}
 
 // S2U (forward) or D2T^T and the transposed closing (adjoint) on the leaves, and the leaf
 // rows' planes
@@ -139,9 +154,7 @@ cudaError_t FarSteps<T>::leaf_in(cudaStream_t s) {
         c2.Y = rows_at<T>(A, ctx, d, nsp), c2.ldy = nsp;
         FMM_CUDA_TRY(gemm<T>(ctx, c2, OP_CLOSE2 + dir * OP_COUNT, s));
     }
-    if (f16)
-        FMM_CUDA_TRY(launch_rows_to_planes((const float *)rows_at<T>(A, ctx, d, nsp), nsp, ctx->lev[d].n, nsp, upP(d),
-                                           ctx->upp_plane, nsp, upS(d), nck_s, s));
+    if (f16) FMM_CUDA_TRY(planes((const float *)rows_at<T>(A, ctx, d, nsp), nsp, d, upP(d), ctx->upp_plane, upS(d), s));
     return cudaSuccess;
 }
 
@@ -153,11 +166,15 @@ cudaError_t FarSteps<T>::up(int l, cudaStream_t s) {
     c.X0 = rows_at<T>(A, ctx, l + 1, nsp), c.ldx0 = nsp, c.k0 = nsp;
     c.W0 = O(l).up[0], c.w_stride = (int64_t)nsp * nsp;
     c.Y = rows_at<T>(A, ctx, l, nsp), c.ldy = nsp;
+    const bool fused = f16 && !O(l).wide;   // one CTA holds a row: it writes the planes too
+    c.xp_chunk_scales = O(l).wide;
     if (f16) {
-        c.Xp = upP(l + 1), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l + 1), c.xp_scale_ld = nck_s;
-        c.Yp = upP(l), c.yp_ld = nsp, c.yp_plane = ctx->upp_plane, c.yp_scale = upS(l), c.yp_scale_ld = nck_s;
+        c.Xp = upP(l + 1), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l + 1);
+        if (fused) c.Yp = upP(l), c.yp_ld = nsp, c.yp_plane = ctx->upp_plane, c.yp_scale = upS(l);
     }
-    return gemm<T>(ctx, c, OP_UP + (adjoint ? OP_COUNT : 0), s);
+    FMM_CUDA_TRY(gemm<T>(ctx, c, OP_UP + (adjoint ? OP_COUNT : 0), s));
+    if (f16 && !fused) FMM_CUDA_TRY(planes((const float *)c.Y, nsp, l, upP(l), ctx->upp_plane, upS(l), s));
+    return cudaSuccess;
 }
 
 // VLI compress: Ut_l = Vi^T U_l.  Tensor-core modes pass the compressed vectors to the stencil
@@ -169,19 +186,34 @@ cudaError_t FarSteps<T>::compress(int l, cudaStream_t s) {
     c.mode = GM_IDENTITY, c.level = l, c.n_out = o.kinp;
     c.X0 = rows_at<T>(A, ctx, l, nsp), c.ldx0 = nsp, c.k0 = nsp, c.W0 = o.compress;
     c.Y = ctx->tensor ? nullptr : rows_at<T>(ctx->Ut, ctx, l, kw), c.ldy = kw;   // tensor modes: planes only
-    if (ctx->tensor) {
-        c.Yp = utP(l), c.yp_ld = kw, c.yp_plane = ctx->utp_plane;
-        c.yp_scale = utS(l), c.yp_scale_ld = nck_k;
+    const bool fused = f16 && !o.wide;
+    c.xp_chunk_scales = o.wide;
+    if (f16) {
+        c.Xp = upP(l), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l);
+        if (!fused) c.Y = rows_at<T>(ctx->Ut, ctx, l, kw);
     }
-    if (f16) c.Xp = upP(l), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l), c.xp_scale_ld = nck_s;
-    return gemm<T>(ctx, c, OP_COMPRESS + (adjoint ? OP_COUNT : 0), s);
+    if (ctx->tensor && (!f16 || fused)) {
+        c.Yp = utP(l), c.yp_ld = kw, c.yp_plane = ctx->utp_plane;
+        c.yp_scale = utS(l);
+    }
+    FMM_CUDA_TRY(gemm<T>(ctx, c, OP_COMPRESS + (adjoint ? OP_COUNT : 0), s));
+    if (f16 && !fused)
+        FMM_CUDA_TRY(launch_rows_planes((const float *)c.Y, 0, 1, kw, nullptr, ctx->lev[l].n, o.kinp, nullptr, 0, utP(l),
+                                        ctx->utp_plane, kw, utS(l), scales(o.kinp), 2, s));
+    return cudaSuccess;
 }
 
 template <typename T> unsigned char *FarSteps<T>::utP(int l) const {
     const int pesz = ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
     return (unsigned char *)ctx->UtP + base(l) * kw * pesz;
 }
-template <typename T> float *FarSteps<T>::utS(int l) const { return ctx->Uscale ? ctx->Uscale + base(l) * nck_k : nullptr; }
+template <typename T> float *FarSteps<T>::utS(int l) const { return ctx->Uscale ? ctx->Uscale + base(l) * (f16 ? scales(O(d).kinp) : 1) : nullptr; }
+
+// rows of level l that can be sources: its boxes and, in a virtual rank's context, its ghosts
+template <typename T> int64_t FarSteps<T>::source_rows(int l) const {
+    const int64_t b = ctx->lev[l].row_base, e = l < d ? ctx->lev[l + 1].row_base : 0;
+    return (e > b ? e : ctx->total_rows) - b;
+}
 
 // VLI stencil: Ct_l[b] = sum_t C_t Ut_l[b + t]
 template <typename T>
@@ -192,15 +224,30 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
     st.X0 = rows_at<T>(ctx->Ut, ctx, l, kw), st.ldx0 = kw, st.k0 = o.kinp;
     st.W0 = o.stencil, st.w_stride = (int64_t)o.koutp * o.kinp;
     st.Y = rows_at<T>(ctx->Ct, ctx, l, kw), st.ldy = kw;
-    if (ctx->tensor) {
+    if (ctx->tensor || ctx->f32m2l) {
         st.Xp = utP(l), st.xp_ld = kw, st.xp_rows = (int)ctx->lev[l].n, st.xp_plane = ctx->utp_plane;
-        st.xp_scale = utS(l), st.xp_scale_ld = nck_k;
+        st.xp_scale = utS(l);
     }
-    if (f16) {   // the decompress reads the stencil output as planes
+    const int op = OP_STENCIL + (adjoint ? OP_COUNT : 0);
+    if (!f16 && !ctx->f32m2l) return gemm<T>(ctx, st, op, s);
+    if (ctx->f32m2l)   // FP32 rows (of the ghosts too) to three planes
+        FMM_CUDA_TRY(launch_rows_planes((const float *)st.X0, 0, 1, kw, nullptr, source_rows(l), o.kinp, nullptr, 0,
+                                        utP(l), ctx->utp_plane, kw, utS(l), 1, 3, s));
+    // FP32 mode reads FP32 rows next; FP16X3 planes, written by the stencil itself if one CTA holds
+    // a row, else from FP32 rows
+    st.groups = stencil_groups(o, l);
+    if (st.groups > 1) st.Y = ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
+    const bool fused = f16 && st.groups == 1 && !o.wide;
+    st.xp_chunk_scales = f16 && o.wide;
+    if (fused) {
         st.Y = nullptr;
-        st.Yp = ctP(l), st.yp_ld = kw, st.yp_plane = ctx->ctp_plane, st.yp_scale = ctS(l), st.yp_scale_ld = nck_k;
+        st.Yp = ctP(l), st.yp_ld = kw, st.yp_plane = ctx->ctp_plane, st.yp_scale = ctS(l);
     }
-    return gemm<T>(ctx, st, OP_STENCIL + (adjoint ? OP_COUNT : 0), s);
+    FMM_CUDA_TRY(gemm<T>(ctx, st, op, s));
+    if (fused || (ctx->f32m2l && st.groups == 1)) return cudaSuccess;
+    return launch_rows_planes((const float *)st.Y, st.y_group, st.groups, kw, nullptr, ctx->lev[l].n, o.koutp,
+                              f16 ? nullptr : (float *)rows_at<T>(ctx->Ct, ctx, l, kw), kw, f16 ? ctP(l) : nullptr,
+                              ctx->ctp_plane, kw, f16 ? ctS(l) : nullptr, f16 ? scales(o.koutp) : 1, 2, s);
 }
 
 // downward step of level l: decompress fused with the parent's D2D contribution (l >= 3)
@@ -215,15 +262,17 @@ cudaError_t FarSteps<T>::down(int l, cudaStream_t s) {
         c.W1_by_cls = O(l - 1).down;
     }
     c.Y = rows_at<T>(B, ctx, l, nsp), c.ldy = nsp;
+    const bool children = l < d;   // the leaves' rows have no children to read them as planes
+    const bool fused = f16 && children && !O(l).wide;
+    c.xp_chunk_scales = O(l).wide;
     if (f16) {
-        c.Xp = ctP(l), c.xp_ld = kw, c.xp_plane = ctx->ctp_plane, c.xp_scale = ctS(l), c.xp_scale_ld = nck_k;
-        if (l >= 3)
-            c.Xp1 = dnP(l - 1), c.xp1_ld = nsp, c.xp1_plane = ctx->upp_plane, c.xp1_scale = dnS(l - 1),
-            c.xp1_scale_ld = nck_s;
-        if (l < d)   // the leaves' rows have no children to read them as planes
-            c.Yp = dnP(l), c.yp_ld = nsp, c.yp_plane = ctx->upp_plane, c.yp_scale = dnS(l), c.yp_scale_ld = nck_s;
+        c.Xp = ctP(l), c.xp_ld = kw, c.xp_plane = ctx->ctp_plane, c.xp_scale = ctS(l);
+        if (l >= 3) c.Xp1 = dnP(l - 1), c.xp1_ld = nsp, c.xp1_plane = ctx->upp_plane, c.xp1_scale = dnS(l - 1);
+        if (fused) c.Yp = dnP(l), c.yp_ld = nsp, c.yp_plane = ctx->upp_plane, c.yp_scale = dnS(l);
     }
     FMM_CUDA_TRY(gemm<T>(ctx, c, OP_DECOMPRESS + (adjoint ? OP_COUNT : 0), s));
+    if (f16 && children && !fused)
+        FMM_CUDA_TRY(planes((const float *)c.Y, nsp, l, dnP(l), ctx->upp_plane, dnS(l), s));
     if (!adjoint && ctx->opt.mean_free) {
         const LevelTables &L = ctx->lev[l];
         double *cm = (double *)ctx->Cmean;
@@ -347,7 +396,7 @@ cudaError_t upload_padded(fmm_ctx *ctx, const std::vector<double> &w, int rows, 
 template <typename T>
 cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
     const int ns = h.ns, nsp = round_up(ns, 16);
-    o.ns = ns, o.nsp = nsp;
+    o.ns = ns, o.nsp = nsp, o.cplx = h.npts != h.ns, o.wide = nsp > 160;
     o.kin = adjoint ? h.kout : h.kin;
     o.kout = adjoint ? h.kin : h.kout;
     o.kinp = round_up(o.kin, 16), o.koutp = round_up(o.kout, 16);
@@ -360,10 +409,23 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
     FMM_CUDA_TRY(upload_padded<T>(ctx, ups, ns, ns, nsp, nsp, 8, &o.up[0]));
     for (int c = 1; c < 8; ++c) o.up[c] = (T *)o.up[0] + (size_t)c * nsp * nsp;
     for (int c = 0; c < 8; ++c) FMM_CUDA_TRY(upload_padded<T>(ctx, down[c], ns, ns, nsp, nsp, 1, &o.down[c]));
+    if (ctx->f16) {
+        std::vector<double> downs;
+        for (int c = 0; c < 8; ++c) downs.insert(downs.end(), down[c].begin(), down[c].end());
+        FMM_CUDA_TRY(f16_upload(ctx, ups.data(), 8, ns, ns, nsp, 2, o.wide, &o.f_up));
+        FMM_CUDA_TRY(f16_upload(ctx, downs.data(), 8, ns, ns, nsp, 2, o.wide, &o.f_down));
+        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_compress : h.compress).data(), 1, o.kin, ns, nsp, 2, o.wide, &o.f_compress));
+        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_decompress : h.decompress).data(), 1, ns, o.kout, o.koutp, 2, o.wide,
+                                &o.f_decompress));
+    }
+    if (ctx->f16 || ctx->f32m2l)
+        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_stencil : h.stencil).data(), kNumTransfer, o.kout, o.kin, o.kinp,
+                                ctx->f16 ? 2 : 3, o.wide, &o.f_stencil));
     if (!h.fft_n) {   // the compressed M2L (the FFT form has its own transforms, fft.cu)
         FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_compress : h.compress, o.kin, ns, o.kinp, nsp, 1, &o.compress));
-        FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_stencil : h.stencil, o.kout, o.kin, o.koutp, o.kinp,
-                                      kNumTransfer, &o.stencil));
+        if (ctx->fp64)   // the others read planes
+            FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_stencil : h.stencil, o.kout, o.kin, o.koutp, o.kinp,
+                                          kNumTransfer, &o.stencil));
         FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_decompress : h.decompress, ns, o.kout, nsp, o.koutp, 1,
                                       &o.decompress));
     }
@@ -399,7 +461,7 @@ cudaError_t upload_operators(fmm_ctx *ctx) {
             FMM_CUDA_TRY(upload_set<float>(ctx, h, true, ctx->adj[l]));
         }
     }
-    if (ctx->tensor) FMM_CUDA_TRY(tc_upload_operators(ctx));
+    if (ctx->tensor && !ctx->f16) FMM_CUDA_TRY(tc_upload_operators(ctx));
     if (ctx->fft) FMM_CUDA_TRY(fft_upload(ctx));
     // unit surface grid in the storage type
     std::vector<double> g = surface_grid(ctx->opt.order_p);

@@ -36,11 +36,25 @@ constexpr int kClassSlots = 189;      // transfer vectors with adjacent parents,
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+// Operators as FP16 planes for gemm_f16.cu (`count` of them, op_bytes apart), each scaled by one
+// power of two: [nsplit][K chunk][plane][16-byte unit of K][ncta output columns][16 B].
+struct F16Mat {
+    void *data = nullptr;
+    float *scale = nullptr;     // 1 / scale per operator, or (two planes, wide) per operator and chunk
+    int n_out = 0;              // output columns (rows of the operator), nsplit * ncta when padded
+    int ncta = 0, nsplit = 0;   // output columns per CTA, CTAs across the columns
+    int K = 0, chunk = 0;       // padded input columns, and per stage
+    int planes = 0;             // 2: hi, lo (22 bits); 3: hi, mid, lo (33 bits)
+    size_t op_bytes = 0;
+};
+
 // Operators of one direction (forward or adjoint) in one arithmetic, device-resident.
 // Row-major [rows x cols] with cols padded: a matrix applied to a padded row vector.
 struct OpSet {
     // host-side shapes
     int ns = 0, nsp = 0;        // surface size and its padding to 16
+    bool cplx = false;          // real form of complex operators (ns = 2 x the surface points)
+    bool wide = false;          // box vectors of more than 160 entries: FP16 planes of two scaled per 64 columns
     int kin = 0, kinp = 0;      // M2L compressed source rank (Vi^T: kin x ns)
     int kout = 0, koutp = 0;    // M2L compressed target rank (Uo: ns x kout)
     int rcl = 0, rclp = 0;      // leaf-closing rank
@@ -58,6 +72,9 @@ struct OpSet {
     int rclu = 0, rclup = 0;
     void *uclose1 = nullptr;    // [rclup x nsp] (U^T)
     void *uclose2 = nullptr;    // [nsp x rclup] (V S^-1)
+    // FP16 planes: FMM_FP16X3 every contraction but the closing (two planes), FMM_FP32 the stencil
+    // (three planes, as accurate as FP32 arithmetic)
+    F16Mat f_up, f_down, f_compress, f_stencil, f_decompress;
 };
 
 // Split operand planes for the tcgen05 GEMMs (gemm_tc.cu): planes[0] holds `count` operators,
@@ -68,8 +85,6 @@ struct TcMat {
     int rows = 0, cols = 0;     // padded N x K
     int nplanes = 0;
     size_t bytes = 0;           // one operator
-    float *scale = nullptr;     // FP16 planes: 1 / (power-of-two scale) per operator and K chunk
-    int scale_ld = 0;           // K chunks per operator
 };
 
 struct TcOpSet {
@@ -130,6 +145,8 @@ struct fmm_ctx {
     bool tensor = false;        // tcgen05 contractions
     bool cplx = false;          // complex densities and outputs (FMM_HELMHOLTZ)
     bool fft = false;           // M2L by FFT (FMM_M2L_FFT)
+    bool f16 = false;           // FMM_FP16X3: contractions from two FP16 planes (gemm_f16.cu)
+    bool f32m2l = false;        // FMM_FP32: stencil from three FP16 planes (gemm_f16.cu)
     void *fft_ghat = nullptr;   // FFT M2L: the kernel's transforms [316][n n (n/2+1)] complex, storage type
     int *fft_surf = nullptr;    // FFT M2L: p^3 grid index of every surface point
     int *fft_tindex = nullptr;  // FFT M2L: transfer index of (neighbour offset, source octant, target octant), -1 near
@@ -182,8 +199,11 @@ struct fmm_ctx {
     void *Yc = nullptr;                  // [nleaf x rclp] closing intermediate
     void *Dq = nullptr;                  // [nleaf x nsp] leaf equivalent densities
     void *Cmean = nullptr;               // [total_rows] FP64 constant part of the downward check potentials
-    float *Uscale = nullptr;             // FMM_FP16X3: 1 / scale of UtP per row and 64-column chunk
-    // FMM_FP16X3: FP16 hi/lo planes (and scales) of the upward-side rows of the current direction
+    float *Uscale = nullptr;             // FMM_FP16X3, FMM_FP32: 1 / scale of every row of UtP
+    float *StP = nullptr;                // ... and the stencil's partial rows of levels 2..5 (stencil_groups)
+    size_t stp_floats = 0;
+    long long stp_base[fmm::kMaxDepth + 1] = {};    // first float of each level's partial rows
+    // FMM_FP16X3: FP16 hi/lo planes (and row scales) of the upward-side rows of the current direction
     // (UpP, [rows x nsp]), of its downward-side rows (DnP) and of the stencil output (CtP, [rows x ws_kw])
     void *UpP = nullptr, *DnP = nullptr, *CtP = nullptr;
     long long upp_plane = 0, ctp_plane = 0;   // bytes per plane (UpP and DnP share the first)
@@ -403,20 +423,32 @@ struct GemmCall {
     // byte (r * ld + k) * esize + p * plane within the buffer (esize 2 for BF16, 4 for TF32).
     const void *Xp = nullptr; int xp_ld = 0; int xp_rows = 0; long long xp_plane = 0;
     void *Yp = nullptr; int yp_ld = 0; long long yp_plane = 0;
-    // FP16 split planes (FMM_FP16X3): 1 / scale per row and 64-column chunk of Xp / Yp
-    const float *xp_scale = nullptr; int xp_scale_ld = 0;
-    float *yp_scale = nullptr; int yp_scale_ld = 0;
-    // PARENT2 segment 1 from split planes (FMM_FP16X3): the parent rows
+    // FP16 planes (gemm_f16): 1 / scale of every row of Xp / Yp (of Xp per 64 columns if
+    // xp_chunk_scales), and the parent rows of PARENT2
+    const float *xp_scale = nullptr; bool xp_chunk_scales = false;
+    float *yp_scale = nullptr;
     const void *Xp1 = nullptr; int xp1_ld = 0; long long xp1_plane = 0;
-    const float *xp1_scale = nullptr; int xp1_scale_ld = 0;
+    const float *xp1_scale = nullptr;
+    // gemm_f16: the transfer vectors cut into `groups`, group z's sums written to Y + z * y_group
+    int groups = 1; long long y_group = 0;
 };
 template <typename T>
 cudaError_t gemm_simt(const fmm_ctx *ctx, const GemmCall &g, cudaStream_t s);
 cudaError_t gemm_tc(const fmm_ctx *ctx, const GemmCall &g, int op_id, cudaStream_t s);
-// FP32 rows (nrows x ncols, stride ldx) -> FP16 hi/lo planes (stride ldp, planes plane_bytes
-// apart) and 1 / scale per row and 64-column chunk (stride lds), as FMM_FP16X3 contractions read
-cudaError_t launch_rows_to_planes(const float *x, int ldx, int64_t nrows, int ncols, void *planes,
-                                  long long plane_bytes, int ldp, float *scales, int lds, cudaStream_t s);
+// gemm_f16.cu: the same contraction from FP16 planes (rows c.Xp / c.Xp1 with one scale each), with
+// the operators W (PARENT2: W for the box's own rows, W1 for its parent's)
+cudaError_t gemm_f16(const fmm_ctx *ctx, const GemmCall &c, const F16Mat &W, const F16Mat *W1, cudaStream_t s);
+// `count` FP64 operators (rows x cols, K the padded cols) packed on the device into `planes` planes
+// (wide: scaled per 64 columns, as their rows)
+cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, int planes, bool wide,
+                       F16Mat *out);
+// rows list[i] (or i) < nrows: sum of `groups` partial rows (x_group apart), to FP32 rows y and / or
+// to FP16 planes with nsc scales a row (one, or one per 64 columns)
+cudaError_t launch_rows_planes(const float *x, long long x_group, int groups, int ldx, const int *list, int64_t nrows,
+                               int ncols, float *y, int ldy, void *planes, long long plane_bytes, int ldp,
+                               float *inv_scale, int nsc, int nplanes, cudaStream_t s);
+// groups of transfer vectors of a level's stencil (gemm_f16)
+int stencil_groups(const OpSet &o, int level);
 cudaError_t tc_upload_operators(fmm_ctx *ctx);
 void tc_free(fmm_ctx *ctx);
 
@@ -435,7 +467,7 @@ template <typename T>
 struct FarSteps {
     fmm_ctx *ctx;
     bool adjoint;
-    int d = 0, nsp = 0, kw = 0, nck_s = 0, nck_k = 0;
+    int d = 0, nsp = 0, kw = 0;
     bool f16 = false;
     void *A = nullptr, *B = nullptr;   // upward- and downward-side rows of this direction
     FarSteps(fmm_ctx *c, bool adj);
@@ -445,6 +477,8 @@ struct FarSteps {
     cudaError_t stencil(int l, cudaStream_t s);          // VLI stencil of level l
     cudaError_t down(int l, cudaStream_t s);             // decompress + D2D into level l
     cudaError_t leaf_out(T *far_phi, T *far_grad, cudaStream_t s);   // closing + D2T
+    cudaError_t planes(const float *x, int n, int l, unsigned char *out, long long plane, float *inv_scale, cudaStream_t s);
+    int64_t source_rows(int l) const;
     size_t base(int l) const { return (size_t)ctx->lev[l].row_base; }
     const OpSet &O(int l) const;
     unsigned char *upP(int l) const;
@@ -455,6 +489,7 @@ struct FarSteps {
     float *dnS(int l) const;
     float *ctS(int l) const;
     float *utS(int l) const;
+    int scales(int cols) const { return O(d).wide ? (cols + 63) / 64 : 1; }   // of a row of FP16 planes (FP16X3)
 };
 
 }  // namespace fmm

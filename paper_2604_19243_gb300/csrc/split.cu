@@ -158,6 +158,7 @@ fmm_ctx *new_view(const fmm_ctx *ctx) {
     v->device = ctx->device;
     v->fp64 = ctx->fp64;
     v->tensor = ctx->tensor;
+    v->f16 = ctx->f16, v->f32m2l = ctx->f32m2l;
     v->ns = ctx->ns, v->nsp = ctx->nsp, v->npts = ctx->npts;
     v->cplx = ctx->cplx;
     for (int a = 0; a < 3; ++a) v->origin[a] = ctx->origin[a];
@@ -565,10 +566,11 @@ fmm_status split_setup(fmm_ctx *ctx, int dg, int P) {
     // exchange tables
     const int nsp = ctx->nsp, kw = S->views[0]->ws_kw;
     const int es = ctx->fp64 ? 8 : 4;
-    const bool f16 = ctx->opt.precision == FMM_FP16X3;
+    const bool f16 = ctx->f16;
+    const OpSet &ops = ctx->fwd[d];
+    const int sc_s = ops.wide ? (nsp + 63) / 64 * 4 : 4, sc_k = ops.wide ? (ops.kinp + 63) / 64 * 4 : 4;   // bytes of a row's scales
     const int np = ctx->opt.precision == FMM_BF16X6 ? 3 : 2;
     const int pesz = ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
-    const int nck_s = (nsp + 63) / 64, nck_k = (kw + 63) / 64;
     std::vector<RowCopy> vex, gat, sca;
     std::vector<PtsCopy> uex;
     S->n_ghost_pts.assign(P, 0);
@@ -616,7 +618,7 @@ fmm_status split_setup(fmm_ctx *ctx, int dg, int P) {
         for (int p = 0; p < np; ++p)
             arr([&](fmm_ctx *v) { return (unsigned char *)v->UtP + p * v->utp_plane; }, (long long)kw * pesz, kw * pesz,
                 S->arr_v);
-        if (f16) arr([&](fmm_ctx *v) { return (unsigned char *)v->Uscale; }, nck_k * 4LL, nck_k * 4, S->arr_v);
+        if (f16) arr([&](fmm_ctx *v) { return (unsigned char *)v->Uscale; }, sc_k, sc_k, S->arr_v);
     }
     arr([&](fmm_ctx *v) { return (unsigned char *)v->Uc; }, (long long)nsp * es, nsp * es, S->arr_up);
     arr([&](fmm_ctx *v) { return (unsigned char *)v->Dc; }, (long long)nsp * es, nsp * es, S->arr_dn);
@@ -625,8 +627,8 @@ fmm_status split_setup(fmm_ctx *ctx, int dg, int P) {
             arr([&](fmm_ctx *v) { return (unsigned char *)v->UpP + p * v->upp_plane; }, nsp * 2LL, nsp * 2, S->arr_up);
             arr([&](fmm_ctx *v) { return (unsigned char *)v->DnP + p * v->upp_plane; }, nsp * 2LL, nsp * 2, S->arr_dn);
         }
-        arr([&](fmm_ctx *v) { return (unsigned char *)v->Ups; }, nck_s * 4LL, nck_s * 4, S->arr_up);
-        arr([&](fmm_ctx *v) { return (unsigned char *)v->Dns; }, nck_s * 4LL, nck_s * 4, S->arr_dn);
+        arr([&](fmm_ctx *v) { return (unsigned char *)v->Ups; }, sc_s, sc_s, S->arr_up);
+        arr([&](fmm_ctx *v) { return (unsigned char *)v->Dns; }, sc_s, sc_s, S->arr_dn);
     }
     if (e == cudaSuccess) {
         std::vector<void *> pb;

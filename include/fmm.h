@@ -59,7 +59,8 @@ typedef enum {
     FMM_FP32 = 0,          /* FP32 SIMT, but for the dense VLI: FP32 values held as three FP16 terms
                               (33 bits) on the tensor cores, FP32 sums; its error against 64 bits is
                               no larger than FP32 arithmetic's */
-    FMM_FP64 = 1,          /* FP64 SIMT everywhere; inputs and outputs are double */
+    FMM_FP64 = 1,          /* FP64; inputs and outputs are double.  SIMT, but for the dense VLI: exact
+                              products of 7-bit digits on the tensor cores (56 bits), FP64 sums */
     FMM_TF32X3 = 2,        /* contractions on tcgen05 tensor cores, 3 TF32 products (big/small split) */
     FMM_BF16X3 = 3,        /* contractions on tcgen05 tensor cores, 3 BF16 products (hi/lo split) */
     FMM_BF16X6 = 4,        /* contractions on tcgen05 tensor cores, 6 BF16 products (hi/mid/lo split) */

@@ -855,21 +855,28 @@ fmm_status adaptive_prepare(fmm_ctx *ctx) {
     return FMM_OK;
 }
 
-// VLI stencil of one level over its kept boxes: FP64 by the SIMT GEMM, FP32 from three FP16 planes
-// on the tensor cores (gemm_f16.cu), in the uniform tree's groups of transfer vectors.
+// VLI stencil of one level over its kept boxes on the tensor cores, as the uniform tree's: FP32 from
+// three FP16 planes (gemm_f16.cu), FP64 from integer digits (gemm_f64.cu).
 template <typename T>
 static cudaError_t adaptive_stencil(fmm_ctx *ctx, GemmCall st, const AdaptiveLevel &L, cudaStream_t s) {
-    if (!ctx->f32m2l) return gemm_simt<T>(ctx, st, s);
     const int l = st.level, kw = ctx->ws_kw;
     const OpSet &o = ctx->fwd[l];
     const size_t rb = (size_t)ctx->lev[l].row_base;
+    if constexpr (sizeof(T) == 8)
+        if (ctx->f64m2l) {
+            st.groups = stencil_groups(o, l);
+            st.y_group = (long long)ctx->lev[l].n * kw;
+            return stencil_f64(ctx, st, o.d_stencil, L.kept, L.n_kept, (unsigned char *)ctx->UtP + rb * kw * kDigitBytes,
+                               (int *)ctx->Uscale + rb, L.kept, L.n_kept, (double *)ctx->StP + ctx->stp_base[l], s);
+        }
+    if (!ctx->f32m2l) return gemm_simt<T>(ctx, st, s);
     st.Xp = (unsigned char *)ctx->UtP + rb * kw * 2, st.xp_ld = kw, st.xp_plane = ctx->utp_plane;
     st.xp_scale = ctx->Uscale + rb;
     FMM_CUDA_TRY(launch_rows_planes((const float *)st.X0, 0, 1, kw, L.kept, L.n_kept, o.kinp, nullptr, 0, (void *)st.Xp,
                                     ctx->utp_plane, kw, ctx->Uscale + rb, 1, 3, s));
     float *ct = (float *)st.Y;
     st.groups = stencil_groups(o, l);
-    if (st.groups > 1) st.Y = ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
+    if (st.groups > 1) st.Y = (float *)ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
     FMM_CUDA_TRY(gemm_f16(ctx, st, o.f_stencil, nullptr, s));
     if (st.groups == 1) return cudaSuccess;
     return launch_rows_planes((const float *)st.Y, st.y_group, st.groups, kw, L.kept, L.n_kept, o.koutp, ct, kw, nullptr,

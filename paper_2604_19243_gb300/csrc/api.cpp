@@ -174,7 +174,7 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
     const int64_t need_rows = ctx->total_rows, need_nl = ctx->nleaf, need_n = ctx->n;
     // partial rows of the stencil's groups (gemm_f16.cu)
     size_t stp = 0;
-    if (ctx->f16 || ctx->f32m2l) {
+    if (ctx->f16 || ctx->f32m2l || ctx->f64m2l) {
         const OpSet &o = ctx->fwd[ctx->opt.depth];
         const int kw = std::max(std::max(o.kinp, o.koutp), 16);
         for (int l = 2; l <= ctx->opt.depth; ++l) {
@@ -182,11 +182,11 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
             if (stencil_groups(o, l) > 1) stp += (size_t)stencil_groups(o, l) * ctx->lev[l].n * kw;
         }
     }
-    if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n || stp > ctx->stp_floats))
+    if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n || stp > ctx->stp_vals))
         free_workspace(ctx);
     if (ctx->have_ws) {
         if (!ctx->tiles_ok) {
-            cudaError_t e = build_tiles(ctx, ctx->fp64 ? 64 : 128);
+            cudaError_t e = build_tiles(ctx, 128);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "tile construction");
             ctx->tiles_ok = true;
         }
@@ -216,15 +216,16 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         {&ctx->near_grad, (size_t)n * 3 * vc * es}, {&ctx->far_phi, (size_t)n * vc * es},
         {&ctx->far_grad, (size_t)n * 3 * vc * es}, {&ctx->pts_qi, ctx->cplx ? (size_t)n * es : (size_t)16},
     };
-    if (ctx->tensor || ctx->f32m2l) {
-        const int np = ctx->opt.precision == FMM_BF16X6 || ctx->f32m2l ? 3 : 2;
-        const size_t pesz = ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
+    if (ctx->tensor || ctx->f32m2l || ctx->f64m2l) {
+        const int np = ctx->f64m2l ? 1 : ctx->opt.precision == FMM_BF16X6 || ctx->f32m2l ? 3 : 2;
+        // (FP64: one array of digit rows)
+        const size_t pesz = ctx->f64m2l ? kDigitBytes : ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
         ctx->utp_plane = (long long)((size_t)rows * kw * pesz + 256) / 256 * 256;
         bool okp = pool_alloc(&ctx->UtP, (size_t)ctx->utp_plane * np, s) == cudaSuccess;
         const size_t nsc = ctx->f16 && o.wide ? (size_t)(std::max(nsp, kw) + 63) / 64 : 1;   // scales a row
-        if (ctx->f16 || ctx->f32m2l)
+        if (ctx->f16 || ctx->f32m2l || ctx->f64m2l)
             okp = okp && pool_alloc((void **)&ctx->Uscale, (size_t)rows * nsc * sizeof(float) + 16, s) == cudaSuccess &&
-                  pool_alloc((void **)&ctx->StP, stp * sizeof(float) + 16, s) == cudaSuccess;
+                  pool_alloc(&ctx->StP, stp * es + 16, s) == cudaSuccess;
         if (ctx->f16) {
             // every contraction reads FP16 planes: the upward- and downward-side rows, the
             // compressed vectors (UtP) and the stencil output, each with its row scales
@@ -243,7 +244,7 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
             free_workspace(ctx);
             return fail(ctx, FMM_ENOMEM, "workspace allocation failed (split planes)");
         }
-        ctx->stp_floats = stp;
+        ctx->stp_vals = stp;
     }
     size_t total = 0;
     for (auto &a : allocs) {
@@ -261,7 +262,7 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         if (p == &ctx->Ut) b = std::max<size_t>(ut_bytes, 16);
         cudaMemsetAsync(*p, 0, b, s);
     }
-    cudaError_t e = build_tiles(ctx, ctx->fp64 ? 64 : 128);
+    cudaError_t e = build_tiles(ctx, 128);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tile construction");
     ctx->tiles_ok = true;
     ctx->ws_bytes = total;

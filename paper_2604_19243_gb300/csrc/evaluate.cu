@@ -229,6 +229,14 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
         st.xp_scale = utS(l);
     }
     const int op = OP_STENCIL + (adjoint ? OP_COUNT : 0);
+    if constexpr (sizeof(T) == 8)
+        if (ctx->f64m2l) {   // (the ghosts' rows too)
+            st.groups = stencil_groups(o, l);
+            st.y_group = (long long)ctx->lev[l].n * kw;
+            return stencil_f64(ctx, st, o.d_stencil, nullptr, source_rows(l),
+                               (unsigned char *)ctx->UtP + base(l) * kw * kDigitBytes, (int *)ctx->Uscale + base(l), nullptr,
+                               ctx->lev[l].n, (double *)ctx->StP + ctx->stp_base[l], s);
+        }
     if (!f16 && !ctx->f32m2l) return gemm<T>(ctx, st, op, s);
     if (ctx->f32m2l)   // FP32 rows (of the ghosts too) to three planes
         FMM_CUDA_TRY(launch_rows_planes((const float *)st.X0, 0, 1, kw, nullptr, source_rows(l), o.kinp, nullptr, 0,
@@ -236,7 +244,7 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
     // FP32 mode reads FP32 rows next; FP16X3 planes, written by the stencil itself if one CTA holds
     // a row, else from FP32 rows
     st.groups = stencil_groups(o, l);
-    if (st.groups > 1) st.Y = ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
+    if (st.groups > 1) st.Y = (float *)ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
     const bool fused = f16 && st.groups == 1 && !o.wide;
     st.xp_chunk_scales = f16 && o.wide;
     if (fused) {
@@ -423,7 +431,10 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
                                 ctx->f16 ? 2 : 3, o.wide, &o.f_stencil));
     if (!h.fft_n) {   // the compressed M2L (the FFT form has its own transforms, fft.cu)
         FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_compress : h.compress, o.kin, ns, o.kinp, nsp, 1, &o.compress));
-        if (ctx->fp64)   // the others read planes
+        if (ctx->f64m2l)
+            FMM_CUDA_TRY(f64_upload(ctx, (adjoint ? h.a_stencil : h.stencil).data(), kNumTransfer, o.kout, o.kin, o.kinp,
+                                    &o.d_stencil));
+        else if (ctx->fp64)   // the others read planes
             FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_stencil : h.stencil, o.kout, o.kin, o.koutp, o.kinp,
                                           kNumTransfer, &o.stencil));
         FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_decompress : h.decompress, ns, o.kout, nsp, o.koutp, 1,
@@ -442,6 +453,10 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
 }  // namespace
 
 cudaError_t upload_operators(fmm_ctx *ctx) {
+    // the digit form of the FP64 stencil needs sums of K products to stay exact, in either direction
+    // (every level's ranks are the same)
+    const HostOps &hd = *ctx->host_ops[ctx->opt.depth];
+    ctx->f64m2l = ctx->fp64 && !ctx->fft && f64_stencil_ok(round_up(std::max(hd.kin, hd.kout), 16));
     // every distinct host set once; levels sharing a set share its device copy
     for (int l = 0; l <= kMaxDepth; ++l) {
         int first = -1;

@@ -31,6 +31,7 @@ constexpr int kMaxDepth = 10;
 // coordinate flag, boxes per child octant per level
 constexpr int kCntLevel = 0, kCntU = kMaxDepth + 1, kCntBad = kMaxDepth + 2, kCntOct = kMaxDepth + 3;
 constexpr int kCntSize = kCntOct + 8 * (kMaxDepth + 1);
+constexpr int kDigitBytes = 16;       // of one FP64 value as integer digits (gemm_f64.cu)
 constexpr int kNumTransfer = 316;     // [-3,3]^3 minus [-1,1]^3
 constexpr int kClassSlots = 189;      // transfer vectors with adjacent parents, per octant
 
@@ -45,6 +46,14 @@ struct F16Mat {
     int ncta = 0, nsplit = 0;   // output columns per CTA, CTAs across the columns
     int K = 0, chunk = 0;       // padded input columns, and per stage
     int planes = 0;             // 2: hi, lo (22 bits); 3: hi, mid, lo (33 bits)
+    size_t op_bytes = 0;
+};
+
+// FP64 operators as integer digits for gemm_f64.cu
+struct F64Mat {
+    void *data = nullptr;
+    int *exps = nullptr;        // binary exponent per operator
+    int K = 0, nsplit = 0;      // padded input columns, CTAs across the output columns
     size_t op_bytes = 0;
 };
 
@@ -75,6 +84,7 @@ struct OpSet {
     // FP16 planes: FMM_FP16X3 every contraction but the closing (two planes), FMM_FP32 the stencil
     // (three planes, as accurate as FP32 arithmetic)
     F16Mat f_up, f_down, f_compress, f_stencil, f_decompress;
+    F64Mat d_stencil;           // FMM_FP64: the stencil as integer digits
 };
 
 // Split operand planes for the tcgen05 GEMMs (gemm_tc.cu): planes[0] holds `count` operators,
@@ -147,6 +157,7 @@ struct fmm_ctx {
     bool fft = false;           // M2L by FFT (FMM_M2L_FFT)
     bool f16 = false;           // FMM_FP16X3: contractions from two FP16 planes (gemm_f16.cu)
     bool f32m2l = false;        // FMM_FP32: stencil from three FP16 planes (gemm_f16.cu)
+    bool f64m2l = false;        // FMM_FP64: stencil from integer digits (gemm_f64.cu; set by the operator upload)
     void *fft_ghat = nullptr;   // FFT M2L: the kernel's transforms [316][n n (n/2+1)] complex, storage type
     int *fft_surf = nullptr;    // FFT M2L: p^3 grid index of every surface point
     int *fft_tindex = nullptr;  // FFT M2L: transfer index of (neighbour offset, source octant, target octant), -1 near
@@ -199,10 +210,10 @@ struct fmm_ctx {
     void *Yc = nullptr;                  // [nleaf x rclp] closing intermediate
     void *Dq = nullptr;                  // [nleaf x nsp] leaf equivalent densities
     void *Cmean = nullptr;               // [total_rows] FP64 constant part of the downward check potentials
-    float *Uscale = nullptr;             // FMM_FP16X3, FMM_FP32: 1 / scale of every row of UtP
-    float *StP = nullptr;                // ... and the stencil's partial rows of levels 2..5 (stencil_groups)
-    size_t stp_floats = 0;
-    long long stp_base[fmm::kMaxDepth + 1] = {};    // first float of each level's partial rows
+    float *Uscale = nullptr;             // FMM_FP16X3, FMM_FP32: 1 / scale of every row of UtP (FMM_FP64: exponents)
+    void *StP = nullptr;                 // ... and the stencil's partial rows of levels 2..5 (stencil_groups)
+    size_t stp_vals = 0;
+    long long stp_base[fmm::kMaxDepth + 1] = {};    // first value of each level's partial rows
     // FMM_FP16X3: FP16 hi/lo planes (and row scales) of the upward-side rows of the current direction
     // (UpP, [rows x nsp]), of its downward-side rows (DnP) and of the stencil output (CtP, [rows x ws_kw])
     void *UpP = nullptr, *DnP = nullptr, *CtP = nullptr;
@@ -447,7 +458,15 @@ cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int c
 cudaError_t launch_rows_planes(const float *x, long long x_group, int groups, int ldx, const int *list, int64_t nrows,
                                int ncols, float *y, int ldy, void *planes, long long plane_bytes, int ldp,
                                float *inv_scale, int nsc, int nplanes, cudaStream_t s);
-// groups of transfer vectors of a level's stencil (gemm_f16)
+// gemm_f64.cu: the FP64 stencil c from integer digits: the source rows (source_list, or the first
+// n_source) to digit_rows and exps (those of c's level), the groups' partial rows in `partial`, summed
+// for the target rows (list, or the first n_rows)
+cudaError_t f64_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, F64Mat *out);
+bool f64_stencil_ok(int K);
+cudaError_t stencil_f64(const fmm_ctx *ctx, const GemmCall &c, const F64Mat &W, const int *source_list, int64_t n_source,
+                        unsigned char *digit_rows, int *exps, const int *list, int64_t n_rows, double *partial,
+                        cudaStream_t s);
+// groups of transfer vectors of a level's stencil (gemm_f16, gemm_f64)
 int stencil_groups(const OpSet &o, int level);
 cudaError_t tc_upload_operators(fmm_ctx *ctx);
 void tc_free(fmm_ctx *ctx);

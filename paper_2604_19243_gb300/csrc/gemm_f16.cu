@@ -646,11 +646,11 @@ int chunk_of(int K, int planes, bool wide) {
 // many CTAs there are, and the number depends on the level alone: the same boxes give the same bits in
 // any partition.
 int stencil_groups(const OpSet &o, int level) {
-    // Real box vectors of more than 160 entries (p >= 7) keep the sums of a box in one sequence: with
+    // Real box vectors of more than 160 entries (p >= 7) in FP32 sums keep the sums of a box in one sequence: with
     // charges of one sign, potentials in a deep tree are thousands of times their variation across a
     // leaf, and another order of the same sums moves the gradients by as much as their own error (4e-5
     // on 4.2M points at depth 6, p = 8).
-    if (o.wide && !o.cplx) return 1;
+    if (o.wide && !o.cplx && !o.d_stencil.data) return 1;
     return level <= 3 ? 19 : level == 4 ? 9 : level == 5 ? 7 : 1;
 }
 

@@ -158,7 +158,7 @@ fmm_ctx *new_view(const fmm_ctx *ctx) {
     v->device = ctx->device;
     v->fp64 = ctx->fp64;
     v->tensor = ctx->tensor;
-    v->f16 = ctx->f16, v->f32m2l = ctx->f32m2l;
+    v->f16 = ctx->f16, v->f32m2l = ctx->f32m2l, v->f64m2l = ctx->f64m2l;
     v->ns = ctx->ns, v->nsp = ctx->nsp, v->npts = ctx->npts;
     v->cplx = ctx->cplx;
     for (int a = 0; a < 3; ++a) v->origin[a] = ctx->origin[a];

@@ -128,6 +128,12 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
+// K-major, SWIZZLE_32B: 32-byte rows, 256 B between 8-row groups, layout type 6.
+__device__ __forceinline__ uint64_t sw32_desc(uint32_t saddr) {
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+
 // K-major descriptor without swizzle: core matrices of 8 rows x 16 bytes, contiguous (128 B) along
 // the rows (SBO = 128 B between 8-row groups), `unit` bytes (LBO) from one 16-byte unit of K to the
 // next.
@@ -195,6 +201,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *r) {
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// 8 consecutive columns of this thread's TMEM lane (no wait)
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
 
 // 16 consecutive columns of this thread's TMEM lane (no wait)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *r) {

@@ -124,11 +124,8 @@ void free_workspace(fmm_ctx *ctx) {
     free_async(ctx->far_phi, s), free_async(ctx->far_grad, s), free_async(ctx->pts_qi, s);
     free_async(ctx->stage_in, s), free_async(ctx->stage_out, s), free_async(ctx->stage_grad, s);
     for (int l = 0; l <= kMaxDepth; ++l)
-        for (TileSet *ts : {&ctx->tiles_plain[l], &ctx->tiles_cls[l]}) {
-            free_async(ts->tiles, s), free_async(ts->masks, s);
-            ts->host.clear();
-            ts->ntiles = 0;
-        }
+        ctx->tiles_plain[l] = TileSet{}, ctx->tiles_cls[l] = TileSet{};
+    free_async(ctx->tiles_all, s), free_async(ctx->masks_all, s);
     ctx->have_ws = false;
     ctx->ws_bytes = 0;
 }
@@ -136,16 +133,15 @@ void free_workspace(fmm_ctx *ctx) {
 // The workspaces outlive the tree: a new tree reuses them when it fits (see ensure_workspace).
 void free_tree(fmm_ctx *ctx) {
     cudaStream_t s = ctx->stream;
+    if (ctx->masks_ev) cudaStreamWaitEvent(s, ctx->masks_ev, 0);   // the side stream reads the tables
     free_async(ctx->pts, s), free_async(ctx->perm, s), free_async(ctx->leaf_off, s), free_async(ctx->inv_perm, s);
     free_async(ctx->u_off, s), free_async(ctx->u_idx, s), free_async(ctx->p2p_order, s);
     for (int l = 0; l <= kMaxDepth; ++l) {
         LevelTables &L = ctx->lev[l];
-        free_async(L.keys, s), free_async(L.parent, s), free_async(L.child, s);
-        free_async(L.dense, s);
         if (!ctx->cls_all) free_async(L.cls_rows, s);
         L = LevelTables{};
     }
-    free_async(ctx->cls_all, s);
+    free_async(ctx->cls_all, s), free_async(ctx->tables, s);
     ctx->have_tree = false;
     ctx->tiles_ok = false;
     ctx->last_far = false;

@@ -141,7 +141,6 @@ struct TileSet {                // tiles of one level for one tile height
     int tile_m = 0;             // rows per tile at most (0: the context's tile_m)
     Tile *tiles = nullptr;      // device
     uint32_t *masks = nullptr;  // device [ntiles x 6] (stencil active-slot bits)
-    std::vector<Tile> host;
 };
 
 }  // namespace fmm
@@ -198,6 +197,11 @@ struct fmm_ctx {
     // class order of every level in one allocation (lev[l].cls_rows point into it); null when
     // each level owns its own array (the contexts of virtual ranks)
     int *cls_all = nullptr;
+    // every level's keys, parent, child and dense tables in one allocation (lev[l] point into it); null
+    // in the contexts of virtual ranks, whose tables the partition owns
+    int *tables = nullptr;
+    fmm::Tile *tiles_all = nullptr;     // every level's tiles (tiles_plain, tiles_cls point into it)
+    uint32_t *masks_all = nullptr;      // every level's stencil masks
 
     // evaluate workspaces (allocated with the tree once operators are known)
     bool have_ws = false;

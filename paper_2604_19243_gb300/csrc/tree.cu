@@ -21,7 +21,8 @@
 namespace fmm {
 
 // ---------------------------------------------------------------------------------------
-// exclusive scan (three-phase: block scans, scan of block sums, add-back)
+// exclusive scan: one launch up to 1024 values, else three (block scans, the block sums scanned by
+// one block, add-back)
 // ---------------------------------------------------------------------------------------
 namespace {
 
@@ -29,10 +30,12 @@ constexpr int kScanThreads = 256;
 constexpr int kScanItems = 4;
 constexpr int kScanBlock = kScanThreads * kScanItems;
 
+// Exclusive scan of d[base .. base + kScanBlock) (zeros past n) plus `add`; returns the block's sum
+// plus `add` in every thread.
 template <typename T>
-__global__ void scan_blocks(T *d, int64_t n, T *block_sums) {
+__device__ __forceinline__ T scan_block(T *d, int64_t base, int64_t n, T add) {
     __shared__ T warp_tot[kScanThreads / 32];
-    const int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanItems;
+    base += (int64_t)threadIdx.x * kScanItems;
     T v[kScanItems];
     T run = 0;
     for (int i = 0; i < kScanItems; ++i) {
@@ -50,37 +53,42 @@ __global__ void scan_blocks(T *d, int64_t n, T *block_sums) {
     }
     if (lane == 31) warp_tot[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        T w = lane < kScanThreads / 32 ? warp_tot[lane] : (T)0;
-        for (int o = 1; o < 32; o <<= 1) {
-            T y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        if (lane < kScanThreads / 32) warp_tot[lane] = w;  // inclusive over warps
+    T before = 0, all = 0;
+    for (int w = 0; w < kScanThreads / 32; ++w) {
+        if (w == warp) before = all;
+        all += warp_tot[w];
     }
-    __syncthreads();
-    T excl = inc - run + (warp > 0 ? warp_tot[warp - 1] : (T)0);
+    __syncthreads();   // warp_tot is reused by the next call
+    const T excl = add + before + inc - run;
     for (int i = 0; i < kScanItems; ++i) {
         int64_t k = base + i;
         if (k < n) d[k] = v[i] + excl;
     }
-    if (threadIdx.x == kScanThreads - 1 && block_sums) block_sums[blockIdx.x] = excl + run;
+    return add + all;
 }
 
 template <typename T>
-__global__ void scan_add(T *d, int64_t n, const T *offsets) {
+__global__ void __launch_bounds__(kScanThreads) scan_blocks(T *d, int64_t n, T *block_sums) {
+    const T sum = scan_block<T>(d, (int64_t)blockIdx.x * kScanBlock, n, (T)0);
+    if (threadIdx.x == 0) block_sums[blockIdx.x] = sum;
+}
+
+// one block scans n values, block after block, and writes their sum (if asked for)
+template <typename T>
+__global__ void __launch_bounds__(kScanThreads) scan_one(T *d, int64_t n, T *total) {
+    T run = 0;
+    for (int64_t b = 0; b < n; b += kScanBlock) run = scan_block<T>(d, b, n, run);
+    if (total && threadIdx.x == 0) *total = run;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kScanThreads) scan_add(T *d, int64_t n, const T *offsets) {
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
     const T add = offsets[blockIdx.x];
     for (int i = threadIdx.x; i < kScanBlock; i += kScanThreads) {
         int64_t k = base + i;
         if (k < n) d[k] += add;
     }
-}
-
-template <typename T>
-__global__ void scan_total(const T *d_scanned, const T *d_orig_last, int64_t n, T *total) {
-    // total = scanned[n-1] + original last value (saved before the scan)
-    *total = n > 0 ? d_scanned[n - 1] + *d_orig_last : (T)0;
 }
 
 }  // namespace
@@ -91,28 +99,17 @@ cudaError_t exclusive_scan(T *d, int64_t n, T *d_total, cudaStream_t s) {
         if (d_total) FMM_CUDA_TRY(cudaMemsetAsync(d_total, 0, sizeof(T), s));
         return cudaSuccess;
     }
-    Scratch<T> last;
-    if (d_total) {
-        FMM_CUDA_TRY(last.alloc(1, s));
-        FMM_CUDA_TRY(cudaMemcpyAsync(last.p, d + n - 1, sizeof(T), cudaMemcpyDeviceToDevice, s));
-    }
-    int64_t nb = (n + kScanBlock - 1) / kScanBlock;
+    const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
     if (nb == 1) {
-        scan_blocks<T><<<1, kScanThreads, 0, s>>>(d, n, nullptr); count_launch();
-    } else {
-        Scratch<T> sums;
-        FMM_CUDA_TRY(sums.alloc(nb, s));
-        scan_blocks<T><<<(unsigned)nb, kScanThreads, 0, s>>>(d, n, sums.p); count_launch();
-        FMM_CUDA_TRY(cudaGetLastError());
-        FMM_CUDA_TRY(exclusive_scan<T>(sums.p, nb, nullptr, s));
-        scan_add<T><<<(unsigned)nb, kScanThreads, 0, s>>>(d, n, sums.p); count_launch();
+        scan_one<T><<<1, kScanThreads, 0, s>>>(d, n, d_total); count_launch();
+        return cudaGetLastError();
     }
-    FMM_CUDA_TRY(cudaGetLastError());
-    if (d_total) {
-        scan_total<T><<<1, 1, 0, s>>>(d, last.p, n, d_total); count_launch();
-        FMM_CUDA_TRY(cudaGetLastError());
-    }
-    return cudaSuccess;
+    Scratch<T> sums;
+    FMM_CUDA_TRY(sums.alloc(nb, s));
+    scan_blocks<T><<<(unsigned)nb, kScanThreads, 0, s>>>(d, n, sums.p); count_launch();
+    scan_one<T><<<1, kScanThreads, 0, s>>>(sums.p, nb, d_total); count_launch();
+    scan_add<T><<<(unsigned)nb, kScanThreads, 0, s>>>(d, n, sums.p); count_launch();
+    return cudaGetLastError();
 }
 template cudaError_t exclusive_scan<int>(int *, int64_t, int *, cudaStream_t);
 template cudaError_t exclusive_scan<long long>(long long *, int64_t, long long *, cudaStream_t);
@@ -228,16 +225,20 @@ __global__ void morton_kernel(const T *xyz, int64_t n, double ox, double oy, dou
 // ---------------------------------------------------------------------------------------
 constexpr int kSortWarps = 8;
 constexpr int kSortThreads = kSortWarps * 32;
-constexpr int kSortRounds = 16;                         // 32-key rounds per warp
-constexpr int kSortWarpItems = 32 * kSortRounds;        // 512 keys per warp
-constexpr int kSortTile = kSortWarps * kSortWarpItems;  // 4096 keys per tile
+// A warp takes its keys in rounds of 32: 16 rounds (tiles of 4096 keys) where there are enough tiles
+// for every SM, 4 (1024) below, since a tile's rounds are a serial chain (22 us for one of 16 rounds on
+// an otherwise idle GPU, 8 us for one of 4).
+template <int R> constexpr int kSortTileOf = kSortWarps * 32 * R;
+constexpr int kSortTile = kSortTileOf<16>;
 
+template <int R>
 __global__ void radix_hist(const uint32_t *keys, int64_t n, int shift, int ntiles, int *hist) {
     __shared__ int cnt[256];
     for (int i = threadIdx.x; i < 256; i += blockDim.x) cnt[i] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    for (int i = threadIdx.x; i < kSortTile; i += blockDim.x) {
+    constexpr int kTile = kSortTileOf<R>;
+    const int64_t base = (int64_t)blockIdx.x * kTile;
+    for (int i = threadIdx.x; i < kTile; i += blockDim.x) {
         int64_t k = base + i;
         if (k < n) atomicAdd(&cnt[(keys[k] >> shift) & 255u], 1);
     }
@@ -245,25 +246,27 @@ __global__ void radix_hist(const uint32_t *keys, int64_t n, int shift, int ntile
     for (int d = threadIdx.x; d < 256; d += blockDim.x) hist[(int64_t)d * ntiles + blockIdx.x] = cnt[d];
 }
 
-// Scatter of one 4096-key tile: the tile is first ordered by digit in shared memory (stable:
+// Scatter of one tile: the tile is first ordered by digit in shared memory (stable:
 // warp, then round, then lane order), then every digit run is written out by consecutive
 // threads to consecutive addresses, so that the global writes are coalesced.
+template <int R>
 __global__ void radix_scatter(const uint32_t *keys, const int *vals, int64_t n, int shift,
                               int ntiles, const int *offs, uint32_t *keys_out, int *vals_out) {
     __shared__ int wcnt[kSortWarps][256];   // per-warp digit counts, then tile positions
     __shared__ int dstart[256];             // tile-local start of each digit's run
     __shared__ int gbase[256];              // global start of this tile's run of each digit
     __shared__ int wsum[kSortThreads / 32];
-    __shared__ uint32_t sk[kSortTile];
-    __shared__ int sv[kSortTile];
+    constexpr int kTile = kSortTileOf<R>, kWarpItems = 32 * R;
+    __shared__ uint32_t sk[kTile];
+    __shared__ int sv[kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < kSortWarps * 256; i += blockDim.x) (&wcnt[0][0])[i] = 0;
     __syncthreads();
-    const int64_t tbase = (int64_t)blockIdx.x * kSortTile;
-    const int64_t wbase = tbase + (int64_t)warp * kSortWarpItems;
-    const int count = n - tbase < (int64_t)kSortTile ? (int)(n - tbase) : kSortTile;
+    const int64_t tbase = (int64_t)blockIdx.x * kTile;
+    const int64_t wbase = tbase + (int64_t)warp * kWarpItems;
+    const int count = n - tbase < (int64_t)kTile ? (int)(n - tbase) : kTile;
     // per-warp digit counts
-    for (int r = 0; r < kSortRounds; ++r) {
+    for (int r = 0; r < R; ++r) {
         int64_t k = wbase + r * 32 + lane;
         if (k < n) atomicAdd(&wcnt[warp][(keys[k] >> shift) & 255u], 1);
     }
@@ -295,7 +298,7 @@ __global__ void radix_scatter(const uint32_t *keys, const int *vals, int64_t n, 
     __syncthreads();
     // tile order in shared memory
     const unsigned lt = (1u << lane) - 1u;
-    for (int r = 0; r < kSortRounds; ++r) {
+    for (int r = 0; r < R; ++r) {
         int64_t k = wbase + r * 32 + lane;
         bool valid = k < n;
         uint32_t key = valid ? keys[k] : 0u;
@@ -326,7 +329,9 @@ __global__ void radix_scatter(const uint32_t *keys, const int *vals, int64_t n, 
 // Stable sort of (keys, vals) by the low `bits` bits of the keys.  Results end in (keys, vals).
 cudaError_t radix_sort(uint32_t *keys, int *vals, int64_t n, int bits, cudaStream_t s) {
     if (n <= 1 || bits <= 0) return cudaSuccess;
-    int ntiles = (int)((n + kSortTile - 1) / kSortTile);
+    const bool small = n < 152 * (int64_t)kSortTile;   // fewer large tiles than SMs
+    const int tile = small ? kSortTileOf<4> : kSortTile;
+    const int ntiles = (int)((n + tile - 1) / tile);
     Scratch<uint32_t> k2;
     Scratch<int> v2, hist;
     FMM_CUDA_TRY(k2.alloc(n, s));
@@ -335,13 +340,15 @@ cudaError_t radix_sort(uint32_t *keys, int *vals, int64_t n, int bits, cudaStrea
     uint32_t *ka = keys, *kb = k2.p;
     int *va = vals, *vb = v2.p;
     int passes = (bits + 7) / 8;
-    for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
-        radix_hist<<<ntiles, kSortThreads, 0, s>>>(ka, n, shift, ntiles, hist.p); count_launch();
+    auto pass = [&](auto h, auto sc, int shift) -> cudaError_t {
+        h<<<ntiles, kSortThreads, 0, s>>>(ka, n, shift, ntiles, hist.p); count_launch();
         FMM_CUDA_TRY(cudaGetLastError());
         FMM_CUDA_TRY(exclusive_scan<int>(hist.p, (int64_t)256 * ntiles, nullptr, s));
-        radix_scatter<<<ntiles, kSortThreads, 0, s>>>(ka, va, n, shift, ntiles, hist.p, kb, vb); count_launch();
-        FMM_CUDA_TRY(cudaGetLastError());
+        sc<<<ntiles, kSortThreads, 0, s>>>(ka, va, n, shift, ntiles, hist.p, kb, vb); count_launch();
+        return cudaGetLastError();
+    };
+    for (int p = 0; p < passes; ++p) {
+        FMM_CUDA_TRY(small ? pass(radix_hist<4>, radix_scatter<4>, 8 * p) : pass(radix_hist<16>, radix_scatter<16>, 8 * p));
         std::swap(ka, kb);
         std::swap(va, vb);
     }
@@ -369,68 +376,116 @@ __global__ void gather_sorted_points(const T *xyz, const int *perm, int64_t n, P
     pts[i] = p;
 }
 
-// Kernels below take the element count either from the host (`cnt` null) or from device
-// memory (`cnt`), with `n` then an upper bound that sizes the grid: the tree build runs from
-// the keys to the U lists without reading a count back.
-__device__ __forceinline__ int64_t count_of(const int *cnt, int64_t n) { return cnt ? (int64_t)*cnt : n; }
+// The boxes of every level from the sorted leaf keys, in one pass over the points.  Point i starts a new
+// box on the levels m(i) .. depth, m(i) the coarsest level on which its key differs from the one
+// before; a box's index on level l is the number of points with m <= l before its first.  level_count
+// counts them per block of 2048 points and level, level_scan scans the blocks of each level, level_fill
+// recounts and writes every table.  Small trees are bound by launches: one pass of flags, scan, compaction,
+// child and dense tables a level took 10 launches a level (70 of the build's 118 at depth 7).  With the
+// smaller sort tiles and the one-pass work order, a step (build and evaluation) went from 519 to 358 us at
+// 20k points, 993 to 725 at 150k, 2430 to 2260 at 1M, 11.60 to 11.39 ms at 8.39M.
+constexpr int kLvThreads = 256, kLvRounds = 8, kLvWarp = 32 * kLvRounds, kLvBlock = 8 * kLvWarp;
 
-// flag[i] = 1 where a new run of (keys >> shift) starts; 0 past the count (up to n)
-__global__ void run_flags(const uint32_t *keys, int64_t n, const int *cnt, int shift, int *flags) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    flags[i] = (i < count_of(cnt, n) && (i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift))) ? 1 : 0;
+struct LevelOut {
+    uint32_t *keys[kMaxDepth + 1];
+    int *parent[kMaxDepth + 1], *child[kMaxDepth + 1], *dense[kMaxDepth + 1];
+};
+
+__device__ __forceinline__ int start_level(const uint32_t *keys, int64_t i, int64_t n, int depth) {
+    if (i >= n) return depth + 1;
+    if (i == 0) return 0;
+    const uint32_t x = keys[i] ^ keys[i - 1];
+    return x == 0u ? depth + 1 : depth - (31 - __clz(x)) / 3;
 }
 
-// After an exclusive scan of the flags: runs get contiguous ids.  For every run start record
-// its position (offsets) and key; for every element record its run id (optional).  The
-// exclusive scan counts the starts strictly before i, so an element that does not start a run
-// sees its own run's start too and its id is the scanned value minus one.
-__global__ void run_compact(const uint32_t *keys, const int *flags_scanned, int64_t n, const int *cnt,
-                            int shift, int *run_start, uint32_t *run_key, int *elem_run) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= count_of(cnt, n)) return;
-    const bool start = (i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift));
-    const int id = flags_scanned[i] - (start ? 0 : 1);
-    if (start) {
-        if (run_start) run_start[id] = (int)i;
-        run_key[id] = keys[i] >> shift;
+// starts of this warp's points per level: lane l returns level l's
+__device__ __forceinline__ int warp_starts(const uint32_t *keys, int64_t w0, int64_t n, int depth, int lane) {
+    int c = 0;
+    for (int r = 0; r < kLvRounds; ++r) {
+        const int m = start_level(keys, w0 + r * 32 + lane, n, depth);
+        for (int l = 0; l <= depth; ++l) {
+            const int k = __popc(__ballot_sync(0xffffffffu, m <= l));
+            if (lane == l) c += k;
+        }
     }
-    if (elem_run) elem_run[i] = id;
+    return c;
 }
 
-// arr[pos] = value, pos from the device when given there
-__global__ void set_last(int *arr, const int *pos_dev, int64_t pos, const int *value_dev, int value) {
-    arr[pos_dev ? *pos_dev : pos] = value_dev ? *value_dev : value;
-}
-
-__global__ void fill_child(const uint32_t *keys, const int *parent, int64_t n, const int *cnt, int *child) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= count_of(cnt, n)) return;
-    child[(int64_t)parent[i] * 8 + (keys[i] & 7u)] = (int)i;
-}
-
-__global__ void fill_dense(const uint32_t *keys, int64_t n, const int *cnt, int *dense) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= count_of(cnt, n)) return;
-    dense[keys[i]] = (int)i;
-}
-
-// boxes per child octant (key & 7) of one level
-__global__ void octant_hist(const uint32_t *keys, int64_t n, const int *cnt, int *hist8) {
-    __shared__ int h[8];
-    if (threadIdx.x < 8) h[threadIdx.x] = 0;
+__global__ void __launch_bounds__(kLvThreads)
+level_count(const uint32_t *__restrict__ keys, int64_t n, int depth, int nblocks, int *__restrict__ cnt) {
+    __shared__ int wc[kLvThreads / 32][kMaxDepth + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = warp_starts(keys, (int64_t)blockIdx.x * kLvBlock + warp * kLvWarp, n, depth, lane);
+    if (lane <= depth) wc[warp][lane] = c;
     __syncthreads();
-    const int64_t c = count_of(cnt, n);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c; i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&h[keys[i] & 7u], 1);
-    __syncthreads();
-    if (threadIdx.x < 8 && h[threadIdx.x]) atomicAdd(&hist8[threadIdx.x], h[threadIdx.x]);
+    if (threadIdx.x <= depth) {
+        int t = 0;
+        for (int w = 0; w < kLvThreads / 32; ++w) t += wc[w][threadIdx.x];
+        cnt[(int64_t)threadIdx.x * nblocks + blockIdx.x] = t;
+    }
 }
 
-// U list of every leaf: its non-empty colleagues and itself, ascending box index (= Morton).
-__global__ void u_count(const uint32_t *keys, int nbound, const int *nleaf, const int *dense, int depth, int *cnt) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nbound) return;
+// block l: exclusive scan of level l's block counts, their sum to totals[l]
+__global__ void __launch_bounds__(kScanThreads) level_scan(int *cnt, int nblocks, int *totals) {
+    int *row = cnt + (int64_t)blockIdx.x * nblocks;
+    int run = 0;
+    for (int b = 0; b < nblocks; b += kScanBlock) run = scan_block<int>(row, b, nblocks, run);
+    if (threadIdx.x == 0) totals[blockIdx.x] = run;
+}
+
+// hist8: boxes per child octant of every level >= 1 (8 a level)
+__global__ void __launch_bounds__(kLvThreads)
+level_fill(const uint32_t *__restrict__ keys, int64_t n, int depth, int nblocks, const int *__restrict__ cnt,
+           LevelOut out, int *__restrict__ leaf_off, int *__restrict__ hist8) {
+    __shared__ int wc[kLvThreads / 32][kMaxDepth + 1];
+    __shared__ int hist[8 * (kMaxDepth + 1)];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w0 = (int64_t)blockIdx.x * kLvBlock + warp * kLvWarp;
+    for (int i = threadIdx.x; i < 8 * (kMaxDepth + 1); i += kLvThreads) hist[i] = 0;
+    const int c = warp_starts(keys, w0, n, depth, lane);
+    if (lane <= depth) wc[warp][lane] = c;
+    __syncthreads();
+    // lane l: starts on level l before this warp's points
+    int run = 0;
+    if (lane <= depth) {
+        run = cnt[(int64_t)lane * nblocks + blockIdx.x];
+        for (int w = 0; w < warp; ++w) run += wc[w][lane];
+    }
+    const unsigned le = 0xffffffffu >> (31 - lane);
+    for (int r = 0; r < kLvRounds; ++r) {
+        const int64_t i = w0 + r * 32 + lane;
+        const int m = start_level(keys, i, n, depth);
+        const uint32_t key = i < n ? keys[i] : 0u;
+        int up = 0;   // box of the point on the level above
+        for (int l = 0; l <= depth; ++l) {
+            const unsigned starts = __ballot_sync(0xffffffffu, m <= l);
+            const int b = __shfl_sync(0xffffffffu, run, l) + __popc(starts & le) - 1;   // its box on level l
+            if (lane == l) run += __popc(starts);
+            if (m <= l) {
+                const uint32_t k = key >> (3 * (depth - l));
+                out.keys[l][b] = k;
+                out.dense[l][k] = b;
+                if (l > 0) {
+                    out.parent[l][b] = up;
+                    out.child[l - 1][(int64_t)up * 8 + (k & 7u)] = b;
+                    atomicAdd(&hist[8 * l + (k & 7u)], 1);
+                }
+                if (l == depth) leaf_off[b] = (int)i;
+            }
+            if (l == depth && i == n - 1) leaf_off[b + 1] = (int)n;
+            up = b;
+        }
+    }
+    __syncthreads();
+    for (int i = 8 + threadIdx.x; i < 8 * (depth + 1); i += kLvThreads)
+        if (hist[i]) atomicAdd(&hist8[i], hist[i]);
+}
+
+// U list of every leaf: its non-empty colleagues and itself, ascending box index (= Morton).  cnt holds
+// nbound + 1 values, zero from the leaf count on.
+__global__ void u_count(const uint32_t *keys, int64_t nbound, const int *nleaf, const int *dense, int depth, int *cnt) {
+    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (b > nbound) return;
     if (b >= *nleaf) {
         cnt[b] = 0;
         return;
@@ -445,48 +500,44 @@ __global__ void u_count(const uint32_t *keys, int nbound, const int *nleaf, cons
     cnt[b] = c;
 }
 
-__global__ void u_fill(const uint32_t *keys, int nleaf, const int *dense, int depth,
-                       const int *off, int *idx) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    int ax, ay, az;
-    demorton3(keys[b], ax, ay, az);
-    int list[27];
-    int c = 0;
-    for (int dx = -1; dx <= 1; ++dx)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dz = -1; dz <= 1; ++dz) {
-                int j = dense_find(dense, depth, ax + dx, ay + dy, az + dz);
-                if (j >= 0) {
-                    int k = c++;   // insertion sort, ascending
-                    while (k > 0 && list[k - 1] > j) {
-                        list[k] = list[k - 1];
-                        --k;
-                    }
-                    list[k] = j;
-                }
-            }
-    for (int k = 0; k < c; ++k) idx[off[b] + k] = list[k];
-}
-
-// work of each leaf for the P2P: |leaf| * sum_{a in U(leaf)} |a|
-__global__ void p2p_work(const int *leaf_off, const int *u_off, const int *u_idx, int nleaf,
-                         uint32_t *work_key, int *order, unsigned long long *total) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    long long src = 0;
-    for (int k = u_off[b]; k < u_off[b + 1]; ++k) {
-        int a = u_idx[k];
-        src += leaf_off[a + 1] - leaf_off[a];
+// One warp per leaf: lane k < 27 looks up neighbour k; its place in the list is the number of smaller
+// indices.  The leaf's near-field work |leaf| * sum_{a in U(leaf)} |a| goes to *total and, as a sort
+// key of 8 bits, to work_key: 255 minus the work's exponent and two mantissa bits (a quarter octave;
+// work < 2^62 fits), so that one ascending pass orders the leaves by decreasing work (equal codes keep
+// Morton order).
+__global__ void __launch_bounds__(256)
+u_fill(const uint32_t *keys, int nleaf, const int *dense, int depth, const int *off, const int *leaf_off, int *idx,
+       uint32_t *work_key, int *order, unsigned long long *total) {
+    __shared__ unsigned long long sum[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x * 8 + warp;
+    long long w = 0;
+    if (b < nleaf) {
+        int ax, ay, az;
+        demorton3(keys[b], ax, ay, az);
+        const int j = lane < 27 ? dense_find(dense, depth, ax + lane / 9 - 1, ay + (lane / 3) % 3 - 1, az + lane % 3 - 1) : -1;
+        int rank = 0, size = j >= 0 ? leaf_off[j + 1] - leaf_off[j] : 0;
+        for (int k = 0; k < 27; ++k) {
+            const int o = __shfl_sync(0xffffffffu, j, k);
+            rank += o >= 0 && o < j;
+        }
+        if (j >= 0) idx[off[b] + rank] = j;
+        long long src = size;
+        for (int o = 16; o > 0; o >>= 1) src += __shfl_xor_sync(0xffffffffu, src, o);
+        const int self = __shfl_sync(0xffffffffu, size, 13);   // offset (0, 0, 0)
+        w = src * (long long)self;
+        if (lane == 0) {
+            const uint32_t code = (__float_as_uint((float)w) >> 21) - (127u << 2);
+            work_key[b] = 255u - min(code, 255u);
+            order[b] = b;
+        }
     }
-    long long w = src * (long long)(leaf_off[b + 1] - leaf_off[b]);
-    atomicAdd(total, (unsigned long long)w);
-    // descending work order through an ascending sort of a 16-bit complement: the top 16 bits
-    // of the work as a float (exponent and 7 mantissa bits, monotone in w), so two radix passes
-    // order the leaves by work to within 1 part in 128 (equal codes keep Morton order)
-    const uint32_t code = __float_as_uint((float)w) >> 16;
-    work_key[b] = 0xffffu - code;
-    order[b] = b;
+    if (lane == 0) sum[warp] = (unsigned long long)w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long t = 0;
+        for (int k = 0; k < 8; ++k) t += sum[k];
+        atomicAdd(total, t);
+    }
 }
 
 // Class keys of the boxes of every level, concatenated level after level: (level, child
@@ -545,28 +596,37 @@ void class_slot_table(std::vector<int> &slots, std::vector<int> &deltas) {
 namespace {
 
 // Per tile: bit s of masks[tile*6 + s/32] is set when some row of the tile has a non-empty
-// source box for class slot s.
-__global__ void tile_masks(const Tile *tiles, int ntiles, const int *cls_rows, const uint32_t *keys,
-                           const int *dense, int level, const int *class_delta, uint32_t *masks) {
+// source box for class slot s.  A warp takes a row at a time, lane s mod 32 slot s.
+__global__ void __launch_bounds__(256)
+tile_masks(const Tile *tiles, int ntiles, const int *cls_rows, const uint32_t *keys, const int *dense, int level,
+           const int *class_delta, uint32_t *masks) {
     __shared__ uint32_t m[6];
-    __shared__ int dlt[kClassSlots][3];
-    const int tid = blockIdx.x;
+    const int tid = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (tid >= ntiles) return;
-    Tile tl = tiles[tid];
+    const Tile tl = tiles[tid];
     if (threadIdx.x < 6) m[threadIdx.x] = 0;
-    for (int s = threadIdx.x; s < kClassSlots; s += blockDim.x) {
-        int dx, dy, dz;
-        unpack_delta(class_delta[tl.cls * kClassSlots + s], dx, dy, dz);
-        dlt[s][0] = dx, dlt[s][1] = dy, dlt[s][2] = dz;
+    int dx[6], dy[6], dz[6];
+#pragma unroll
+    for (int w = 0; w < 6; ++w) {
+        const int s = 32 * w + lane;
+        dx[w] = 0, dy[w] = 0, dz[w] = 0;
+        if (s < kClassSlots) unpack_delta(class_delta[tl.cls * kClassSlots + s], dx[w], dy[w], dz[w]);
     }
     __syncthreads();
-    for (int w = threadIdx.x; w < tl.nrows * kClassSlots; w += blockDim.x) {
-        int r = w / kClassSlots, s = w % kClassSlots;
-        int box = cls_rows[tl.row0 + r];
+    uint32_t hit = 0;   // bit w: slot 32 w + lane has a source for one of this warp's rows
+    for (int r = warp; r < tl.nrows; r += 8) {
         int ax, ay, az;
-        demorton3(keys[box], ax, ay, az);
-        if (dense_find(dense, level, ax + dlt[s][0], ay + dlt[s][1], az + dlt[s][2]) >= 0)
-            atomicOr(&m[s >> 5], 1u << (s & 31));
+        demorton3(keys[cls_rows[tl.row0 + r]], ax, ay, az);
+#pragma unroll
+        for (int w = 0; w < 6; ++w)
+            if (32 * w + lane < kClassSlots && !((hit >> w) & 1u) &&
+                dense_find(dense, level, ax + dx[w], ay + dy[w], az + dz[w]) >= 0)
+                hit |= 1u << w;
+    }
+#pragma unroll
+    for (int w = 0; w < 6; ++w) {
+        const uint32_t b = __ballot_sync(0xffffffffu, (hit >> w) & 1u);
+        if (lane == 0 && b) atomicOr(&m[w], b);
     }
     __syncthreads();
     if (threadIdx.x < 6) masks[tid * 6 + threadIdx.x] = m[threadIdx.x];
@@ -709,58 +769,42 @@ static cudaError_t build_tree_t(fmm_ctx *ctx, const T *xyz) {
         gather_sorted_points<T, float4><<<blocks_for(n, 256), 256, 0, s>>>(xyz, ctx->perm, n, (float4 *)ctx->pts);
     count_launch();
     FMM_CUDA_TRY(cudaGetLastError());
-    // 4. leaves (runs of equal keys) and the boxes of every level (runs of equal parent keys)
-    {
-        Scratch<int> flags;
-        FMM_CUDA_TRY(flags.alloc(n, s));
-        run_flags<<<blocks_for(n, 256), 256, 0, s>>>(keys.p, n, nullptr, 0, flags.p); count_launch();
-        FMM_CUDA_TRY(exclusive_scan<int>(flags.p, n, cnt + kCntLevel + depth, s));
-        const int64_t bd = bound(depth);
-        FMM_CUDA_TRY(pool_alloc((void **)&ctx->leaf_off, (bd + 1) * sizeof(int), s));
-        FMM_CUDA_TRY(pool_alloc((void **)&ctx->lev[depth].keys, bd * sizeof(uint32_t), s));
-        run_compact<<<blocks_for(n, 256), 256, 0, s>>>(keys.p, flags.p, n, nullptr, 0, ctx->leaf_off,
-                                                         ctx->lev[depth].keys, nullptr); count_launch();
-        set_last<<<1, 1, 0, s>>>(ctx->leaf_off, cnt + kCntLevel + depth, 0, nullptr, (int)n); count_launch();
-        FMM_CUDA_TRY(cudaGetLastError());
-    }
-    for (int l = depth; l >= 1; --l) {
-        LevelTables &C = ctx->lev[l], &P = ctx->lev[l - 1];
-        const int64_t bc = bound(l), bp = bound(l - 1);
-        const int *nc = cnt + kCntLevel + l;
-        Scratch<int> f;
-        FMM_CUDA_TRY(f.alloc(bc, s));
-        run_flags<<<blocks_for(bc, 256), 256, 0, s>>>(C.keys, bc, nc, 3, f.p); count_launch();
-        FMM_CUDA_TRY(exclusive_scan<int>(f.p, bc, cnt + kCntLevel + l - 1, s));
-        FMM_CUDA_TRY(pool_alloc((void **)&P.keys, bp * sizeof(uint32_t), s));
-        FMM_CUDA_TRY(pool_alloc((void **)&C.parent, bc * sizeof(int), s));
-        run_compact<<<blocks_for(bc, 256), 256, 0, s>>>(C.keys, f.p, bc, nc, 3, nullptr, P.keys, C.parent); count_launch();
-        FMM_CUDA_TRY(pool_alloc((void **)&P.child, (size_t)bp * 8 * sizeof(int), s));
-        FMM_CUDA_TRY(cudaMemsetAsync(P.child, 0xff, (size_t)bp * 8 * sizeof(int), s));
-        fill_child<<<blocks_for(bc, 256), 256, 0, s>>>(C.keys, C.parent, bc, nc, P.child); count_launch();
-        FMM_CUDA_TRY(cudaGetLastError());
-    }
-    // 5. dense tables and the octant histograms
-    for (int l = 0; l <= depth; ++l) {
-        LevelTables &T_ = ctx->lev[l];
-        const int64_t bl = bound(l);
-        size_t sz = (size_t)1 << (3 * l);
-        FMM_CUDA_TRY(pool_alloc((void **)&T_.dense, sz * sizeof(int), s));
-        FMM_CUDA_TRY(cudaMemsetAsync(T_.dense, 0xff, sz * sizeof(int), s));
-        fill_dense<<<blocks_for(bl, 256), 256, 0, s>>>(T_.keys, bl, cnt + kCntLevel + l, T_.dense); count_launch();
-        if (l >= 1) {
-            octant_hist<<<std::min<unsigned>(blocks_for(bl, 256), 256), 256, 0, s>>>(T_.keys, bl, cnt + kCntLevel + l,
-                                                                                       cnt + kCntOct + 8 * l); count_launch();
-        }
-        FMM_CUDA_TRY(cudaGetLastError());
-    }
-    // 6. U-list sizes and offsets
+    // 4-5. leaves, the boxes of every level, their parent, child and dense tables, the octant counts.
+    // The tables of all levels are one allocation, the child and dense tables (empty entries -1) last.
     const int64_t bd = bound(depth);
+    FMM_CUDA_TRY(pool_alloc((void **)&ctx->leaf_off, (bd + 1) * sizeof(int), s));
+    {
+        size_t head = 0, tail = 0;
+        for (int l = 0; l <= depth; ++l) {
+            head += 2 * (size_t)bound(l);
+            tail += ((size_t)1 << (3 * l)) + (l < depth ? 8 * (size_t)bound(l) : 0);
+        }
+        FMM_CUDA_TRY(pool_alloc((void **)&ctx->tables, (head + tail) * sizeof(int), s));
+        FMM_CUDA_TRY(cudaMemsetAsync(ctx->tables + head, 0xff, tail * sizeof(int), s));
+        LevelOut out{};
+        int *h = ctx->tables, *t = ctx->tables + head;
+        for (int l = 0; l <= depth; ++l) {
+            LevelTables &T_ = ctx->lev[l];
+            out.keys[l] = T_.keys = (uint32_t *)h, h += bound(l);
+            out.parent[l] = h, h += bound(l);
+            T_.parent = l > 0 ? out.parent[l] : nullptr;
+            out.dense[l] = T_.dense = t, t += (size_t)1 << (3 * l);
+            if (l < depth) out.child[l] = T_.child = t, t += 8 * (size_t)bound(l);
+        }
+        const int nblk = (int)((n + kLvBlock - 1) / kLvBlock);
+        Scratch<int> lc;
+        FMM_CUDA_TRY(lc.alloc((size_t)(depth + 1) * nblk, s));
+        level_count<<<nblk, kLvThreads, 0, s>>>(keys.p, n, depth, nblk, lc.p); count_launch();
+        level_scan<<<depth + 1, kScanThreads, 0, s>>>(lc.p, nblk, cnt + kCntLevel); count_launch();
+        level_fill<<<nblk, kLvThreads, 0, s>>>(keys.p, n, depth, nblk, lc.p, out, ctx->leaf_off, cnt + kCntOct); count_launch();
+        FMM_CUDA_TRY(cudaGetLastError());
+    }
+    // 6. U-list sizes and offsets (the entry past the last leaf becomes the total)
     FMM_CUDA_TRY(pool_alloc((void **)&ctx->u_off, (bd + 1) * sizeof(int), s));
-    u_count<<<blocks_for(bd, 128), 128, 0, s>>>(ctx->lev[depth].keys, (int)bd, cnt + kCntLevel + depth,
-                                                 ctx->lev[depth].dense, depth, ctx->u_off); count_launch();
+    u_count<<<blocks_for(bd + 1, 128), 128, 0, s>>>(ctx->lev[depth].keys, bd, cnt + kCntLevel + depth,
+                                                     ctx->lev[depth].dense, depth, ctx->u_off); count_launch();
     FMM_CUDA_TRY(cudaGetLastError());
-    FMM_CUDA_TRY(exclusive_scan<int>(ctx->u_off, bd, cnt + kCntU, s));
-    set_last<<<1, 1, 0, s>>>(ctx->u_off, cnt + kCntLevel + depth, 0, cnt + kCntU, 0); count_launch();
+    FMM_CUDA_TRY(exclusive_scan<int>(ctx->u_off, bd + 1, cnt + kCntU, s));
     // the one read-back of the build
     int *hc = ctx->host_counts;
     FMM_CUDA_TRY(cudaMemcpyAsync(hc, cnt, kCntSize * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -779,20 +823,16 @@ static cudaError_t build_tree_t(fmm_ctx *ctx, const T *xyz) {
     const int nleaf = (int)ctx->lev[depth].n;
     ctx->nleaf = nleaf;
     ctx->n_u = hc[kCntU];
-    // U lists
+    // U lists, the P2P schedule (decreasing work) and the total pair count (read when asked for)
     FMM_CUDA_TRY(pool_alloc((void **)&ctx->u_idx, std::max<int64_t>(ctx->n_u, 1) * sizeof(int), s));
-    u_fill<<<blocks_for(nleaf, 128), 128, 0, s>>>(ctx->lev[depth].keys, nleaf, ctx->lev[depth].dense, depth,
-                                                   ctx->u_off, ctx->u_idx); count_launch();
-    FMM_CUDA_TRY(cudaGetLastError());
-    // P2P schedule (decreasing work) and the total pair count (read when asked for)
     {
         Scratch<uint32_t> wk;
         FMM_CUDA_TRY(wk.alloc(nleaf, s));
         FMM_CUDA_TRY(pool_alloc((void **)&ctx->p2p_order, std::max(nleaf, 1) * sizeof(int), s));
-        p2p_work<<<blocks_for(nleaf, 256), 256, 0, s>>>(ctx->leaf_off, ctx->u_off, ctx->u_idx, nleaf,
-                                                          wk.p, ctx->p2p_order, ctx->dev_pairs); count_launch();
+        u_fill<<<blocks_for(nleaf, 8), 256, 0, s>>>(ctx->lev[depth].keys, nleaf, ctx->lev[depth].dense, depth, ctx->u_off,
+                                                    ctx->leaf_off, ctx->u_idx, wk.p, ctx->p2p_order, ctx->dev_pairs); count_launch();
         FMM_CUDA_TRY(cudaGetLastError());
-        FMM_CUDA_TRY(radix_sort(wk.p, ctx->p2p_order, nleaf, 16, s));
+        FMM_CUDA_TRY(radix_sort(wk.p, ctx->p2p_order, nleaf, 8, s));
         ctx->p2p_pairs = -1;
     }
     // class (octant) order of every level at once: one stable sort of all boxes by (level,
@@ -825,39 +865,28 @@ cudaError_t build_tree(fmm_ctx *ctx, const void *d_xyz) {
 cudaError_t build_tiles(fmm_ctx *ctx, int tile_m) {
     cudaStream_t s = ctx->stream;
     const int depth = ctx->opt.depth;
+    // every level's tiles in one device array (plain order, then class order), filled by one copy
     std::vector<Tile> staged;
-    struct Copy {
-        Tile *dst;
-        int count;
-    };
-    std::vector<Copy> copies;
+    if (ctx->masks_ev) FMM_CUDA_TRY(cudaStreamWaitEvent(s, ctx->masks_ev, 0));   // earlier masks of the side stream
+    if (ctx->tiles_all) cudaFreeAsync(ctx->tiles_all, s);
+    if (ctx->masks_all) cudaFreeAsync(ctx->masks_all, s);
+    ctx->tiles_all = nullptr, ctx->masks_all = nullptr;
+    size_t at[kMaxDepth + 1][2] = {}, mask_tiles = 0;
     for (int l = 0; l <= depth; ++l) {
-        for (TileSet *ts : {&ctx->tiles_plain[l], &ctx->tiles_cls[l]}) {
-            if (ts->tiles) cudaFreeAsync(ts->tiles, s);
-            if (ts->masks) cudaFreeAsync(ts->masks, s);
-            ts->tiles = nullptr;
-            ts->masks = nullptr;
-            ts->host.clear();
-            ts->ntiles = 0;
-        }
         LevelTables &T_ = ctx->lev[l];
-        // plain order
-        TileSet &pl = ctx->tiles_plain[l];
+        TileSet &pl = ctx->tiles_plain[l], &cl = ctx->tiles_cls[l];
+        pl = TileSet{}, cl = TileSet{};
+        at[l][0] = staged.size();
         for (int64_t r = 0; r < T_.n; r += tile_m)
-            pl.host.push_back(Tile{(int)r, (int)std::min<int64_t>(tile_m, T_.n - r), -1, 0});
-        // class order
-        TileSet &cl = ctx->tiles_cls[l];
+            staged.push_back(Tile{(int)r, (int)std::min<int64_t>(tile_m, T_.n - r), -1, 0});
+        pl.ntiles = (int)(staged.size() - at[l][0]);
+        at[l][1] = staged.size();
         if (l >= 1)
             for (int c = 0; c < 8; ++c)
                 for (int r = T_.cls_off[c]; r < T_.cls_off[c + 1]; r += tile_m)
-                    cl.host.push_back(Tile{r, std::min(tile_m, T_.cls_off[c + 1] - r), c, (int)cl.host.size()});
-        for (TileSet *ts : {&pl, &cl}) {
-            ts->ntiles = (int)ts->host.size();
-            if (!ts->ntiles) continue;
-            FMM_CUDA_TRY(pool_alloc((void **)&ts->tiles, ts->ntiles * sizeof(Tile), s));
-            staged.insert(staged.end(), ts->host.begin(), ts->host.end());
-            copies.push_back({ts->tiles, ts->ntiles});
-        }
+                    staged.push_back(Tile{r, std::min(tile_m, T_.cls_off[c + 1] - r), c, (int)(staged.size() - at[l][1])});
+        cl.ntiles = (int)(staged.size() - at[l][1]);
+        if (l >= 2) mask_tiles += cl.ntiles;
     }
     if (!ctx->tiles_ev) FMM_CUDA_TRY(cudaEventCreateWithFlags(&ctx->tiles_ev, cudaEventDisableTiming));
     FMM_CUDA_TRY(cudaEventSynchronize(ctx->tiles_ev));   // earlier copies out of the staging buffer
@@ -868,20 +897,25 @@ cudaError_t build_tiles(fmm_ctx *ctx, int tile_m) {
         FMM_CUDA_TRY(cudaMallocHost((void **)&ctx->host_tiles, staged.size() * 2 * sizeof(Tile)));
         ctx->host_tiles_cap = staged.size() * 2;
     }
-    std::copy(staged.begin(), staged.end(), ctx->host_tiles);
-    size_t off = 0;
-    for (const Copy &c : copies) {
-        FMM_CUDA_TRY(cudaMemcpyAsync(c.dst, ctx->host_tiles + off, c.count * sizeof(Tile), cudaMemcpyHostToDevice, s));
-        off += c.count;
+    if (!staged.empty()) {
+        std::copy(staged.begin(), staged.end(), ctx->host_tiles);
+        FMM_CUDA_TRY(pool_alloc((void **)&ctx->tiles_all, staged.size() * sizeof(Tile), s));
+        FMM_CUDA_TRY(cudaMemcpyAsync(ctx->tiles_all, ctx->host_tiles, staged.size() * sizeof(Tile), cudaMemcpyHostToDevice, s));
     }
     FMM_CUDA_TRY(cudaEventRecord(ctx->tiles_ev, s));
+    if (mask_tiles) FMM_CUDA_TRY(pool_alloc((void **)&ctx->masks_all, mask_tiles * 6 * sizeof(uint32_t), s));
+    mask_tiles = 0;
+    for (int l = 0; l <= depth; ++l) {
+        ctx->tiles_plain[l].tiles = ctx->tiles_all + at[l][0];
+        ctx->tiles_cls[l].tiles = ctx->tiles_all + at[l][1];
+        if (l >= 2) {
+            ctx->tiles_cls[l].masks = ctx->masks_all + mask_tiles * 6;
+            mask_tiles += ctx->tiles_cls[l].ntiles;
+        }
+    }
     // The stencil masks are needed only by the VLI, after the upward pass: they are computed on a
     // side stream (aux[1]) while the evaluation starts, and every stencil contraction waits for
     // masks_ev first.
-    for (int l = 2; l <= depth; ++l) {
-        TileSet &cl = ctx->tiles_cls[l];
-        if (cl.ntiles) FMM_CUDA_TRY(pool_alloc((void **)&cl.masks, (size_t)cl.ntiles * 6 * sizeof(uint32_t), s));
-    }
     // (a context without the side stream, a virtual rank's, computes them in stream order)
     const bool side = ctx->aux[1] && ctx->masks_fork_ev && ctx->masks_ev;
     cudaStream_t ms = side ? ctx->aux[1] : s;
@@ -1165,15 +1199,15 @@ cudaError_t noalloc_scratch(unsigned char **out) {
     return cudaSuccess;
 }
 
-// Exclusive scan of n <= kScanBlock * kScanBlock ints with the given block-sum buffer.
+// Exclusive scan of n ints with the given block-sum buffer.
 cudaError_t scan_fixed(int *d, int64_t n, int *sums, cudaStream_t s) {
     const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
     if (nb == 1) {
-        scan_blocks<int><<<1, kScanThreads, 0, s>>>(d, n, nullptr); count_launch();
+        scan_one<int><<<1, kScanThreads, 0, s>>>(d, n, nullptr); count_launch();
         return cudaGetLastError();
     }
     scan_blocks<int><<<(unsigned)nb, kScanThreads, 0, s>>>(d, n, sums); count_launch();
-    scan_blocks<int><<<1, kScanThreads, 0, s>>>(sums, nb, nullptr); count_launch();
+    scan_one<int><<<1, kScanThreads, 0, s>>>(sums, nb, nullptr); count_launch();
     scan_add<int><<<(unsigned)nb, kScanThreads, 0, s>>>(d, n, sums); count_launch();
     return cudaGetLastError();
 }
@@ -1217,9 +1251,9 @@ extern "C" fmm_status fmm_sort_points_noalloc(const float *xyz, int64_t n, int d
     uint32_t *ka = keys, *kb = k2;
     int *va = perm, *vb = v2;
     for (int pass = 0; pass < (bits + 7) / 8 && n > 1; ++pass) {
-        radix_hist<<<ntiles, kSortThreads, 0, s>>>(ka, n, 8 * pass, ntiles, hist); count_launch();
+        radix_hist<16><<<ntiles, kSortThreads, 0, s>>>(ka, n, 8 * pass, ntiles, hist); count_launch();
         if (scan_fixed(hist, (int64_t)256 * ntiles, sums, s) != cudaSuccess) return FMM_ECUDA;
-        radix_scatter<<<ntiles, kSortThreads, 0, s>>>(ka, va, n, 8 * pass, ntiles, hist, kb, vb); count_launch();
+        radix_scatter<16><<<ntiles, kSortThreads, 0, s>>>(ka, va, n, 8 * pass, ntiles, hist, kb, vb); count_launch();
         std::swap(ka, kb);
         std::swap(va, vb);
     }

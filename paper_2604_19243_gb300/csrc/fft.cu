@@ -99,90 +99,136 @@ fft_fwd_kernel(FftShape sh, const T *__restrict__ u, int ldu, const int *__restr
 
 // ĉ[β] = sum over the V list of β of Ĝ_t ⊙ û[α], for this chunk's frequencies.  The V list of a
 // child of parent P is the children of P's 26 neighbours that are not adjacent to it, and the
-// transfer vector of (target octant c, neighbour offset o, source octant c') is 2o + c' - c in
-// child units, the same for every parent (table `pairs`: index t of Ĝ_t, or -1 when adjacent).
-// A CTA takes kHadG consecutive parents and one slice of 32 consecutive frequencies: Ĝ of the
-// slice for all 316 transfer vectors is staged in shared memory; warp g owns parent g, lane j
-// frequency j of the slice, and the thread keeps the 8 children's sums in registers.  Each
-// source value is then read from memory once per parent and applied to all 8 targets.
-constexpr int kHadG = 16;          // parents (warps) per CTA
+// transfer vector of (target octant c, neighbour offset o, source octant c') is d = 2o + c' - c in
+// child units, the same for every parent.  A CTA takes 16 NP consecutive parents and one slice of 32
+// consecutive frequencies; lane j of a warp owns frequency j, the warp NP parents, whose 8 children's
+// sums stay in registers.  Ĝ of the slice lies in shared memory by the cell of d in [-3, 3]^3, so that
+// the 8 targets of a source octant read it at constant distances from one address.
+// What bounds it: 8 bytes of Ĝ feed 4 FMAs, and shared memory delivers a warp's 256 bytes in two cycles
+// in which the SM does 8 warps' FMAs.  One parent a warp (with an index load and a branch a term, and
+// six operations a complex product) ran at 18 % of the FMA rate; with NP = 4 a Ĝ value is used for 16 FMAs.
+// 32768 boxes, p = 8: 7.55 -> 3.36 ms (49 % of the FMA rate; packed FMAs free issue slots but take the
+// same time).  The next source values are loaded while the present ones are multiplied.  Source octants are the outer
+// loop: the 64 parents' sources of one octant are 216 rows where the tree is full, which stay in L1 for
+// the 26 offsets (13312 loads of a CTA, 1728 different rows).
+// FP64 values are twice as large: NP = 2.
+constexpr int kHadG = 16;          // warps per CTA
 constexpr int kHadF = 32;          // frequencies per CTA
+constexpr int kHadCells = 343;     // d in [-3, 3]^3
+template <typename T> constexpr int kHadP = sizeof(T) == 4 ? 4 : 2;   // parents per warp
+template <typename T> constexpr size_t kHadSmem =
+    (size_t)kHadCells * kHadF * sizeof(typename C2<T>::type) + (size_t)kHadG * kHadP<T> * 208 * sizeof(int);
+
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 
 template <typename T>
-__global__ void __launch_bounds__(kHadG * 32)
-fft_hadamard_kernel(const typename C2<T>::type *__restrict__ uh, long long row, int nfreq,
+__global__ void __launch_bounds__(kHadG * 32, 1)
+fft_hadamard_kernel(const typename C2<T>::type *__restrict__ uh, int row, int nfreq,
                     const typename C2<T>::type *__restrict__ ghat, long long ghat_stride,
                     const uint32_t *__restrict__ pkeys, const int *__restrict__ pdense, const int *__restrict__ pchild,
-                    int plevel, int nparent, const int *__restrict__ pairs, typename C2<T>::type *__restrict__ ch) {
+                    int plevel, int nparent, const int *__restrict__ cell_t, typename C2<T>::type *__restrict__ ch) {
     using V = typename C2<T>::type;
-    extern __shared__ unsigned char fft_smem[];
-    V *gs = reinterpret_cast<V *>(fft_smem);   // [316][32]: Ĝ_t of this slice
-    __shared__ int src[kHadG][26][8];          // children of each parent's neighbours (-1: none)
-    __shared__ int tgt[kHadG][8];              // children of each parent
-    __shared__ int tt[26 * 8 * 8];             // transfer index of (o, c', c), -1 when adjacent
+    constexpr int NP = kHadP<T>;
+    extern __shared__ __align__(16) unsigned char fft_smem[];
+    V *gs = reinterpret_cast<V *>(fft_smem);                   // [343][32]: Ĝ of this slice (near cells unused)
+    int *src = reinterpret_cast<int *>(gs + kHadCells * kHadF);   // [warp][c', o][NP]: source box or -1
+    __shared__ int cell0[208];                                 // (c', o): cell of 2o + c'; bits 16..23: near targets c
     const int tid = threadIdx.x, g = tid >> 5, lane = tid & 31;
-    const int p0 = blockIdx.x * kHadG, f0 = blockIdx.y * kHadF, f = f0 + lane;
+    const int p0 = blockIdx.x * (kHadG * NP), f0 = blockIdx.y * kHadF, f = f0 + lane;
     const bool fl = f < nfreq;
-    for (int i = tid; i < 26 * 64; i += blockDim.x) tt[i] = pairs[i];
     constexpr int kU = 8;   // staging loads in flight per thread
-    for (int i0 = tid; i0 < kNumTransfer * kHadF; i0 += kU * kHadG * 32) {
+    for (int i0 = tid; i0 < kHadCells * kHadF; i0 += kU * kHadG * 32) {
         V v[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-            const int i = i0 + u * kHadG * 32, t = i / kHadF, j = i % kHadF;
-            v[u] = (i < kNumTransfer * kHadF && f0 + j < nfreq) ? ghat[(long long)t * ghat_stride + f0 + j]
-                                                                : V{(T)0, (T)0};
+            const int i = i0 + u * kHadG * 32, j = i % kHadF;
+            const int t = i < kHadCells * kHadF ? cell_t[i / kHadF] : -1;
+            v[u] = (t >= 0 && f0 + j < nfreq) ? ghat[(long long)t * ghat_stride + f0 + j] : V{(T)0, (T)0};
         }
 #pragma unroll
         for (int u = 0; u < kU; ++u)
-            if (i0 + u * kHadG * 32 < kNumTransfer * kHadF) gs[i0 + u * kHadG * 32] = v[u];
+            if (i0 + u * kHadG * 32 < kHadCells * kHadF) gs[i0 + u * kHadG * 32] = v[u];
     }
-    for (int e = tid; e < kHadG * 8; e += blockDim.x) {
-        const int gg = e / 8, c = e % 8, P = p0 + gg;
-        tgt[gg][c] = P < nparent ? pchild[(size_t)P * 8 + c] : -1;
+    for (int e = tid; e < 208; e += blockDim.x) {
+        const int oi = e % 26, c2 = e / 26, o = oi < 13 ? oi : oi + 1;   // offsets of [-1,1]^3 without the centre
+        const int x = 2 * (o / 9 - 1) + (c2 >> 2), y = 2 * ((o / 3) % 3 - 1) + ((c2 >> 1) & 1), z = 2 * (o % 3 - 1) + (c2 & 1);
+        int near = 0;
+        for (int c = 0; c < 8; ++c)
+            if (max(abs(x - (c >> 2)), max(abs(y - ((c >> 1) & 1)), abs(z - (c & 1)))) <= 1) near |= 1 << c;
+        cell0[e] = ((x + 3) * 7 + y + 3) * 7 + z + 3 | near << 16;
     }
-    for (int e = tid; e < kHadG * 26; e += blockDim.x) {
-        const int gg = e / 26, oi = e % 26, P = p0 + gg;
-        const int o = oi < 13 ? oi : oi + 1;   // offsets of [-1,1]^3 without the centre
+    for (int e = tid; e < kHadG * NP * 26; e += blockDim.x) {
+        const int q = e / 26, oi = e % 26, P = p0 + q;   // q = warp NP + parent
+        const int o = oi < 13 ? oi : oi + 1;
         int nb = -1;
         if (P < nparent) {
             int ax, ay, az;
             demorton3(pkeys[P], ax, ay, az);
             nb = dense_find(pdense, plevel, ax + o / 9 - 1, ay + (o / 3) % 3 - 1, az + o % 3 - 1);
         }
-        for (int c = 0; c < 8; ++c) src[gg][oi][c] = nb >= 0 ? pchild[(size_t)nb * 8 + c] : -1;
+        for (int c = 0; c < 8; ++c)
+            src[((q / NP) * 208 + c * 26 + oi) * NP + q % NP] = nb >= 0 ? pchild[(size_t)nb * 8 + c] : -1;
     }
     __syncthreads();
-    if (p0 + g >= nparent) return;
-    V acc[8];
+    const int pw = p0 + g * NP;
+    if (pw >= nparent) return;
+    const int *sw = src + g * 208 * NP;
+    V acc[NP][8], next[NP];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = {(T)0, (T)0};
-    for (int oi = 0; oi < 26; ++oi) {
-        V u[8];
+    for (int k = 0; k < NP; ++k)
 #pragma unroll
-        for (int c2 = 0; c2 < 8; ++c2) {
-            const int sb = src[g][oi][c2];
-            u[c2] = (sb >= 0 && fl) ? uh[(long long)sb * row + f] : V{(T)0, (T)0};
+        for (int c = 0; c < 8; ++c) acc[k][c] = {(T)0, (T)0};
+    const V *uf = uh + f;
+    bool some = false;   // whether any parent has the next source
+    auto load = [&](int it) {
+        some = false;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const int sb = sw[it * NP + k];
+            some |= sb >= 0;
+            next[k] = (sb >= 0 && fl) ? uf[(long long)sb * row] : V{(T)0, (T)0};
         }
+    };
+    load(0);
+#pragma unroll 1
+    for (int it = 0; it < 208; ++it) {
+        V u[NP];
 #pragma unroll
-        for (int c2 = 0; c2 < 8; ++c2) {
-            if (src[g][oi][c2] < 0) continue;
-            const int *tp = tt + (oi * 8 + c2) * 8;
+        for (int k = 0; k < NP; ++k) u[k] = next[k];
+        const bool now = some;
+        if (it + 1 < 208) load(it + 1);
+        if (!now) continue;
+        const int cell = cell0[it], near = cell >> 16;
+        const V *gp = gs + (cell & 0xffff) * kHadF + lane;
+        auto term = [&](int c) {
+            const V gv = gp[-(49 * (c >> 2) + 7 * ((c >> 1) & 1) + (c & 1)) * kHadF];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int t = tp[c];
-                if (t < 0) continue;   // adjacent to the target: near field, not V
-                const V gv = gs[t * kHadF + lane];
-                acc[c].x += gv.x * u[c2].x - gv.y * u[c2].y;
-                acc[c].y += gv.x * u[c2].y + gv.y * u[c2].x;
+            for (int k = 0; k < NP; ++k) {
+                acc[k][c].x = fma_(gv.x, u[k].x, acc[k][c].x);
+                acc[k][c].y = fma_(gv.x, u[k].y, acc[k][c].y);
+                acc[k][c].x = fma_(-gv.y, u[k].y, acc[k][c].x);
+                acc[k][c].y = fma_(gv.y, u[k].x, acc[k][c].y);
             }
+        };
+        if (near == 0) {   // 152 of the 208: no test between the targets, so that their Ĝ load together
+#pragma unroll
+            for (int c = 0; c < 8; ++c) term(c);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (!((near >> c) & 1)) term(c);   // the others are adjacent: near field, not V
         }
     }
     if (!fl) return;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const int tb = tgt[g][c];
-        if (tb >= 0) ch[(long long)tb * row + f] = acc[c];
+    for (int k = 0; k < NP; ++k) {
+        if (pw + k >= nparent) break;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int tb = pchild[(size_t)(pw + k) * 8 + c];
+            if (tb >= 0) ch[(long long)tb * row + f] = acc[k][c];
+        }
     }
 }
 
@@ -288,28 +334,17 @@ cudaError_t fft_upload(fmm_ctx *ctx) {
     ctx->op_allocs.push_back(ctx->fft_surf);
     FMM_CUDA_TRY(cudaMemcpy(ctx->fft_surf, surf.data(), surf.size() * sizeof(int), cudaMemcpyHostToDevice));
     // transfer index of every (dx, dy, dz) in [-3, 3]^3 (the order of the kernel transforms:
-    // lexicographic, the near range |d| <= 1 left out), -1 in the near range; then the index of
-    // (neighbour offset o, source octant c', target octant c) with d = 2o + c' - c
-    std::vector<int> tix(343, -1);
+    // lexicographic, the near range |d| <= 1 left out), -1 in the near range
+    std::vector<int> tix(kHadCells, -1);
     int t = 0;
     for (int i = -3; i <= 3; ++i)
         for (int j = -3; j <= 3; ++j)
             for (int k = -3; k <= 3; ++k)
                 if (std::max(std::abs(i), std::max(std::abs(j), std::abs(k))) > 1) tix[((i + 3) * 7 + j + 3) * 7 + k + 3] = t++;
     if (t != kNumTransfer) return cudaErrorInvalidValue;
-    std::vector<int> pairs(26 * 64);
-    for (int oi = 0; oi < 26; ++oi) {
-        const int o = oi < 13 ? oi : oi + 1, ox = o / 9 - 1, oy = (o / 3) % 3 - 1, oz = o % 3 - 1;
-        for (int c2 = 0; c2 < 8; ++c2)
-            for (int c = 0; c < 8; ++c) {
-                const int dx = 2 * ox + ((c2 >> 2) & 1) - ((c >> 2) & 1), dy = 2 * oy + ((c2 >> 1) & 1) - ((c >> 1) & 1),
-                          dz = 2 * oz + (c2 & 1) - (c & 1);
-                pairs[(oi * 8 + c2) * 8 + c] = tix[((dx + 3) * 7 + dy + 3) * 7 + dz + 3];
-            }
-    }
-    FMM_CUDA_TRY(dev_malloc((void **)&ctx->fft_tindex, pairs.size() * sizeof(int)));
+    FMM_CUDA_TRY(dev_malloc((void **)&ctx->fft_tindex, tix.size() * sizeof(int)));
     ctx->op_allocs.push_back(ctx->fft_tindex);
-    FMM_CUDA_TRY(cudaMemcpy(ctx->fft_tindex, pairs.data(), pairs.size() * sizeof(int), cudaMemcpyHostToDevice));
+    FMM_CUDA_TRY(cudaMemcpy(ctx->fft_tindex, tix.data(), tix.size() * sizeof(int), cudaMemcpyHostToDevice));
     return cudaSuccess;
 }
 
@@ -351,7 +386,7 @@ cudaError_t fft_vli(fmm_ctx *ctx, int l, const T *U, T *D, cudaStream_t s) {
     const size_t fs = fwd_smem<T>(sh), is = inv_smem<T>(sh);
     if (fs > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(fft_fwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs));
     if (is > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(fft_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)is));
-    const size_t hs = (size_t)kNumTransfer * kHadF * sizeof(V);
+    const size_t hs = kHadSmem<T>;
     FMM_CUDA_TRY(cudaFuncSetAttribute(fft_hadamard_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
     for (int ka0 = 0; ka0 < sh.n; ka0 += nka) {
         const int k = std::min(nka, sh.n - ka0);
@@ -359,8 +394,8 @@ cudaError_t fft_vli(fmm_ctx *ctx, int l, const T *U, T *D, cudaStream_t s) {
         count_launch();
         FMM_CUDA_TRY(cudaGetLastError());
         const LevelTables &P = ctx->lev[l - 1];
-        const dim3 hg((unsigned)((P.n + kHadG - 1) / kHadG), (unsigned)((k * per + kHadF - 1) / kHadF));
-        fft_hadamard_kernel<T><<<hg, kHadG * 32, hs, s>>>(uh.p, (long long)k * per, k * per, ghat + (size_t)ka0 * per,
+        const dim3 hg((unsigned)((P.n + kHadG * kHadP<T> - 1) / (kHadG * kHadP<T>)), (unsigned)((k * per + kHadF - 1) / kHadF));
+        fft_hadamard_kernel<T><<<hg, kHadG * 32, hs, s>>>(uh.p, k * per, k * per, ghat + (size_t)ka0 * per,
                                                           (long long)sh.n * per, P.keys, P.dense, P.child, l - 1,
                                                           (int)P.n, ctx->fft_tindex, ch.p);
         count_launch();

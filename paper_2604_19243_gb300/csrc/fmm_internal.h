@@ -159,7 +159,7 @@ struct fmm_ctx {
     bool f64m2l = false;        // FMM_FP64: stencil from integer digits (gemm_f64.cu; set by the operator upload)
     void *fft_ghat = nullptr;   // FFT M2L: the kernel's transforms [316][n n (n/2+1)] complex, storage type
     int *fft_surf = nullptr;    // FFT M2L: p^3 grid index of every surface point
-    int *fft_tindex = nullptr;  // FFT M2L: transfer index of (neighbour offset, source octant, target octant), -1 near
+    int *fft_tindex = nullptr;  // FFT M2L: transfer index of every cell of [-3, 3]^3, -1 near
     int npts = 0;               // surface points, 6(p-1)^2+2
     int ns = 0, nsp = 0;        // box vector length (npts, or 2 npts: real then imaginary parts), padded
 

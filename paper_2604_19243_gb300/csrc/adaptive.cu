@@ -297,9 +297,12 @@ __device__ inline void box_centre(uint32_t key, double ox, double oy, double oz,
 
 // XLI (Algorithm 1, step 2b): the sources of every leaf in X(b) on the downward check surface
 // (1.05) of b, added to b's downward check potentials.  One block per box of the level with a
-// non-empty X list (`list`, the level's box indices).
+// non-empty X list (`list`, the level's box indices), one thread per surface point: a second pass for
+// the 24 points of 152 past 128 threads cost as much as the first (507 -> 416 us over three levels).
+constexpr int kXliThreads = (kMaxSurface + 31) / 32 * 32;
+
 template <typename T>
-__global__ void __launch_bounds__(kEvalThreads)
+__global__ void __launch_bounds__(kXliThreads)
 xli_kernel(const typename Pt4<T>::type *__restrict__ pts, const uint32_t *__restrict__ keys, int base,
            const int *__restrict__ x_off, const int *__restrict__ x_idx, const int *__restrict__ begin,
            const int *__restrict__ count, const T *__restrict__ grid, int ns, double ox, double oy, double oz,
@@ -311,7 +314,7 @@ xli_kernel(const typename Pt4<T>::type *__restrict__ pts, const uint32_t *__rest
     if (m0 == m1) return;
     double c[3];
     box_centre(keys[b], ox, oy, oz, width, c);
-    for (int i0 = 0; i0 < ns; i0 += kEvalThreads) {
+    for (int i0 = 0; i0 < ns; i0 += blockDim.x) {
         const int i = i0 + threadIdx.x;
         T px = 0, py = 0, pz = 0, acc = 0;
         if (i < ns) {
@@ -324,7 +327,7 @@ xli_kernel(const typename Pt4<T>::type *__restrict__ pts, const uint32_t *__rest
             for (int c0 = s0; c0 < s1; c0 += kEvalChunk) {
                 const int c1 = min(s1, c0 + kEvalChunk);
                 __syncthreads();
-                for (int e = c0 + threadIdx.x; e < c1; e += kEvalThreads) src[e - c0] = pts[e];
+                for (int e = c0 + threadIdx.x; e < c1; e += blockDim.x) src[e - c0] = pts[e];
                 __syncthreads();
                 if (i < ns)
                     for (int e = 0; e < c1 - c0; ++e) {
@@ -342,6 +345,20 @@ xli_kernel(const typename Pt4<T>::type *__restrict__ pts, const uint32_t *__rest
 // WLI (Algorithm 1, step 3a): the upward equivalent densities (1.05 surface) of every box in
 // W(b) evaluated at the points of leaf b, added to the far-field outputs.  One block per row with
 // a non-empty W list (`list`).
+// The block's warps share out the list: a warp takes every fourth box, keeps its surface in its own part
+// of shared memory and sums it at up to 64 points of the leaf, two a lane; leaves of up to 16 and 8
+// points have 2 and 4 groups of lanes share the surface.  (With one thread a point, leaves of some 30
+// points left three warps of four idle.)  A surface point is (c + r g) rounded once: in FP32 from the
+// centre and radius as sums of two FP32 numbers, since nine FP64 operations a point took longer than
+// the sums; a lane works out the centre of one box of 32 in FP64.
+// 1.05M points of an uneven cloud, p = 6: 2.73 -> 0.67 ms.
+constexpr int kWliWarps = kEvalThreads / 32, kWliChunk = 160;
+
+__device__ __forceinline__ float surface_point(float hi, float lo, float rhi, float rlo, float g) {
+    return hi + fmaf(rhi, g, fmaf(rlo, g, lo));
+}
+__device__ __forceinline__ double surface_point(double hi, double, double rhi, double, double g) { return hi + rhi * g; }
+
 template <typename T, bool GRAD>
 __global__ void __launch_bounds__(kEvalThreads)
 wli_kernel(const typename Pt4<T>::type *__restrict__ pts, Levels L, const int *__restrict__ w_off,
@@ -349,49 +366,88 @@ wli_kernel(const typename Pt4<T>::type *__restrict__ pts, Levels L, const int *_
            const T *__restrict__ grid, int ns, double ox, double oy, double oz, double side,
            const T *__restrict__ ue, int ldu, T *__restrict__ phi, T *__restrict__ grad, const int *__restrict__ list) {
     using P = typename Pt4<T>::type;
-    __shared__ P src[kMaxSurface];
+    __shared__ P surf[kWliWarps][kWliChunk];
+    __shared__ P red[kWliWarps][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = list[blockIdx.x];
     const int m0 = w_off[r], m1 = w_off[r + 1];
     if (m0 == m1) return;
     const int t0 = begin[r], t1 = t0 + count[r];
-    for (int i0 = t0; i0 < t1; i0 += kEvalThreads) {
-        const int i = i0 + threadIdx.x;
-        const P x = pts[min(i, t1 - 1)];
-        T pot = 0, gx = 0, gy = 0, gz = 0;
-        for (int m = m0; m < m1; ++m) {
-            const int a = w_idx[m], la = row_level(L, a);
-            const double width = side / (double)(1 << la), radius = 1.05 * 0.5 * width;
-            double c[3];
-            box_centre(L.keys[la][a - L.base[la]], ox, oy, oz, width, c);
-            __syncthreads();
-            for (int j = threadIdx.x; j < ns; j += kEvalThreads) {
-                P y;
-                y.x = (T)(c[0] + radius * (double)grid[3 * j]);
-                y.y = (T)(c[1] + radius * (double)grid[3 * j + 1]);
-                y.z = (T)(c[2] + radius * (double)grid[3 * j + 2]);
-                y.w = ue[(size_t)a * ldu + j];
-                src[j] = y;
+    P *src = surf[warp];
+    for (int i0 = t0; i0 < t1; i0 += 64) {
+        const int nt = min(64, t1 - i0);
+        const int groups = nt <= 8 ? 4 : nt <= 16 ? 2 : 1, span = 32 / groups;   // lanes a group
+        const int ti = lane & (span - 1), sub = lane / span;
+        const P xa = pts[i0 + min(ti, nt - 1)], xb = pts[i0 + min(ti + 32, nt - 1)];
+        T sa[4] = {0, 0, 0, 0}, sb[4] = {0, 0, 0, 0};   // potential and gradient at the two points
+        auto add = [](const P &x, const P &y, T (&s)[4]) {
+            const T dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z;
+            const T ri = inv_sqrt<T>(dx * dx + dy * dy + dz * dz), w = y.w * ri;
+            s[0] += w;
+            if (GRAD) {
+                const T w3 = w * ri * ri;
+                s[1] -= w3 * dx, s[2] -= w3 * dy, s[3] -= w3 * dz;
             }
-            __syncthreads();
-            for (int j = 0; j < ns; ++j) {
-                const P y = src[j];
-                const T dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z;
-                const T ri = inv_sqrt<T>(dx * dx + dy * dy + dz * dz), w = y.w * ri;
-                pot += w;
-                if (GRAD) {
-                    const T w3 = w * ri * ri;
-                    gx -= w3 * dx, gy -= w3 * dy, gz -= w3 * dz;
+        };
+        for (int mb = m0 + warp; mb < m1; mb += kWliWarps * 32) {
+            const int nm = min(32, (m1 - mb + kWliWarps - 1) / kWliWarps);   // boxes mb, mb + 4, ...
+            int row = 0;
+            T hi[3] = {0, 0, 0}, lo[3] = {0, 0, 0}, rhi = 0, rlo = 0;
+            if (lane < nm) {
+                row = w_idx[mb + lane * kWliWarps];
+                const int la = row_level(L, row);
+                const double width = side / (double)(1 << la), radius = 1.05 * 0.5 * width;
+                double c[3];
+                box_centre(L.keys[la][row - L.base[la]], ox, oy, oz, width, c);
+                for (int k = 0; k < 3; ++k) hi[k] = (T)c[k], lo[k] = (T)(c[k] - (double)hi[k]);
+                rhi = (T)radius, rlo = (T)(radius - (double)rhi);
+            }
+            for (int m = 0; m < nm; ++m) {
+                const unsigned all = 0xffffffffu;
+                const T *u = ue + (size_t)__shfl_sync(all, row, m) * ldu;
+                const T hx = __shfl_sync(all, hi[0], m), hy = __shfl_sync(all, hi[1], m), hz = __shfl_sync(all, hi[2], m);
+                const T lx = __shfl_sync(all, lo[0], m), ly = __shfl_sync(all, lo[1], m), lz = __shfl_sync(all, lo[2], m);
+                const T rh = __shfl_sync(all, rhi, m), rl = __shfl_sync(all, rlo, m);
+                for (int j0 = 0; j0 < ns; j0 += kWliChunk) {
+                    const int nj = min(kWliChunk, ns - j0);
+                    __syncwarp();   // the last chunk has been read
+                    for (int j = lane; j < nj; j += 32) {
+                        const T *g = grid + 3 * (j0 + j);
+                        P y;
+                        y.x = surface_point(hx, lx, rh, rl, g[0]);
+                        y.y = surface_point(hy, ly, rh, rl, g[1]);
+                        y.z = surface_point(hz, lz, rh, rl, g[2]);
+                        y.w = u[j0 + j];
+                        src[j] = y;
+                    }
+                    __syncwarp();
+                    if (nt > 32)
+                        for (int j = 0; j < nj; ++j) add(xa, src[j], sa), add(xb, src[j], sb);
+                    else
+                        for (int j = sub; j < nj; j += groups) add(xa, src[j], sa);
                 }
             }
         }
-        if (i < t1) {
-            if (phi) phi[i] += pot * one_over_4pi<T>();
-            if (GRAD) {
-                grad[3 * (size_t)i] += gx * one_over_4pi<T>();
-                grad[3 * (size_t)i + 1] += gy * one_over_4pi<T>();
-                grad[3 * (size_t)i + 2] += gz * one_over_4pi<T>();
+        for (int o = span; o < 32; o <<= 1)
+            for (int k = 0; k < 4; ++k) sa[k] += __shfl_xor_sync(0xffffffffu, sa[k], o);
+        P v;
+        v.x = sa[0], v.y = sa[1], v.z = sa[2], v.w = sa[3];
+        red[warp][lane] = v;
+        v.x = sb[0], v.y = sb[1], v.z = sb[2], v.w = sb[3];
+        red[warp][lane + 32] = v;
+        __syncthreads();
+        if (threadIdx.x < nt) {
+            const int i = i0 + threadIdx.x;
+            T s[4] = {0, 0, 0, 0};
+            for (int w = 0; w < kWliWarps; ++w) {
+                const P q = red[w][threadIdx.x];
+                s[0] += q.x, s[1] += q.y, s[2] += q.z, s[3] += q.w;
             }
+            if (phi) phi[i] += s[0] * one_over_4pi<T>();
+            if (GRAD)
+                for (int k = 0; k < 3; ++k) grad[3 * (size_t)i + k] += s[1 + k] * one_over_4pi<T>();
         }
+        __syncthreads();
     }
 }
 
@@ -760,7 +816,7 @@ cudaError_t adaptive_xli(const fmm_ctx *ctx, int level, T *D, int ld, cudaStream
     const AdaptiveLevel &L = A->lv[level];
     if (L.n_x == 0) return cudaSuccess;
     const double width = ctx->side / (double)(1 << level);
-    xli_kernel<T><<<(unsigned)L.n_x, kEvalThreads, 0, s>>>(
+    xli_kernel<T><<<(unsigned)L.n_x, std::min((ctx->npts + 31) / 32 * 32, kXliThreads), 0, s>>>(
         (const typename Pt4<T>::type *)ctx->pts, T_.keys, (int)T_.row_base, A->off[3], A->idx[3], A->begin, A->count,
         (const T *)ctx->grid_dev, ctx->npts, ctx->origin[0], ctx->origin[1], ctx->origin[2], width, 1.05 * 0.5 * width,
         D, ld, L.xlist);
@@ -773,7 +829,6 @@ cudaError_t adaptive_wli(fmm_ctx *ctx, T *phi, T *grad, cudaStream_t s) {
     AdaptiveState *A = ctx->adaptive;
     const int D = ctx->opt.depth;
     if (A->n_w == 0 || D < 2) return cudaSuccess;
-    if (ctx->npts > kMaxSurface) return cudaErrorInvalidValue;   // p <= 10 is checked at fmm_create
     const int nsp = ctx->nsp;
     // upward equivalent densities of the kept boxes of levels 2..D: r_l (V S^-1)(U^T U_l)
     for (int l = 2; l <= D; ++l) {

@@ -670,27 +670,18 @@ leaf_eval_kernel(const typename Vec4<T>::type *__restrict__ pts, Boxes bx, const
     extern __shared__ unsigned char smem_raw[];
     P *src = reinterpret_cast<P *>(smem_raw);    // [ns]
     __shared__ double cen[3];
-    __shared__ float cenf[3];
     const int b = list ? list[blockIdx.x] : (int)blockIdx.x;
     if (threadIdx.x == 0) {   // the box centre once per leaf
         int ax, ay, az;
         demorton3(keys[b], ax, ay, az);
         cen[0] = ox + (ax + 0.5) * width, cen[1] = oy + (ay + 0.5) * width, cen[2] = oz + (az + 0.5) * width;
-        cenf[0] = (float)cen[0], cenf[1] = (float)cen[1], cenf[2] = (float)cen[2];
     }
     __syncthreads();
     for (int j = threadIdx.x; j < ns; j += kLeafThreads) {
         P p;
-        if constexpr (std::is_same<T, float>::value) {   // FP32: no FP64 arithmetic per surface point
-            const float r32 = (float)radius;
-            p.x = fmaf(r32, grid[3 * j], cenf[0]);
-            p.y = fmaf(r32, grid[3 * j + 1], cenf[1]);
-            p.z = fmaf(r32, grid[3 * j + 2], cenf[2]);
-        } else {
-            p.x = (T)(cen[0] + radius * (double)grid[3 * j]);
-            p.y = (T)(cen[1] + radius * (double)grid[3 * j + 1]);
-            p.z = (T)(cen[2] + radius * (double)grid[3 * j + 2]);
-        }
+        p.x = (T)(cen[0] + radius * (double)grid[3 * j]);
+        p.y = (T)(cen[1] + radius * (double)grid[3 * j + 1]);
+        p.z = (T)(cen[2] + radius * (double)grid[3 * j + 2]);
         p.w = dens[(int64_t)b * ldd + j];
         src[j] = p;
     }
@@ -698,32 +689,6 @@ leaf_eval_kernel(const typename Vec4<T>::type *__restrict__ pts, Boxes bx, const
     int t0, tn;
     box_range(bx, b, t0, tn);
     const int t1 = t0 + tn;
-    if constexpr (std::is_same<T, float>::value) {
-        // FP32: the (even) surface count re-staged as pairs, two-wide FP32 arithmetic; the
-        // surface lies outside the leaf box, so no distance is zero
-        float4 *pr = reinterpret_cast<float4 *>(smem_raw) + ns;   // [ns] float4 = ns / 2 pairs
-        float *sf = reinterpret_cast<float *>(pr);
-        for (int j = threadIdx.x; j < ns; j += kLeafThreads) {
-            const float4 v = src[j];
-            float *o = sf + 8 * (j >> 1) + (j & 1);
-            o[0] = v.x, o[2] = v.y, o[4] = v.z, o[6] = v.w;
-        }
-        __syncthreads();
-        for (int i = t0 + threadIdx.x; i < t1; i += kLeafThreads) {
-            const float4 x = pts[i];
-            const float2 nx = make_float2(-x.x, -x.x), ny = make_float2(-x.y, -x.y), nz = make_float2(-x.z, -x.z);
-            float2 pot = make_float2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
-            for (int e = 0; e < ns / 2; ++e) pair_step<1, false, YUK>(pr, e, &nx, &ny, &nz, &pot, &gx, &gy, &gz, kappa);
-            const float f = scale * inv4pi<float>();
-            if (phi) phi[i] = (pot.x + pot.y) * f + (shift ? (float)shift[b] : 0.f);   // the leaf's constant part
-            if (GRAD) {
-                grad[3 * (int64_t)i] = (gx.x + gx.y) * f;
-                grad[3 * (int64_t)i + 1] = (gy.x + gy.y) * f;
-                grad[3 * (int64_t)i + 2] = (gz.x + gz.y) * f;
-            }
-        }
-        return;
-    }
     for (int i = t0 + threadIdx.x; i < t1; i += kLeafThreads) {
         const P x = pts[i];
         T pot = 0, gx = 0, gy = 0, gz = 0;
@@ -736,6 +701,88 @@ leaf_eval_kernel(const typename Vec4<T>::type *__restrict__ pts, Boxes bx, const
             grad[3 * (int64_t)i + 2] = gz * f;
         }
     }
+}
+
+// FP32 D2T: a block takes the points of `nl` leaves, a thread each, so that leaves of fewer points than a
+// block has threads fill its warps (one leaf a block left three warps of four idle at 16 points a leaf).  A
+// leaf's surface is staged once, in pairs (the count is even) for the two-wide FP32 arithmetic; the leaves'
+// parts start 32 bytes past a multiple of 128, so that a warp's lanes on two leaves read different banks.
+// The surface lies outside the leaf box, so no distance is zero.
+// 262144 leaves of 16 points, p = 8: 1.68 -> 0.99 ms; 32768 of 30.5, p = 6: 132 -> 103 us; 74722 of 112, p = 6
+// (one leaf a block as before): 0.69 -> 0.71 ms.
+constexpr int kEvalLeaves = 8;
+
+__host__ __device__ __forceinline__ int eval_stride(int ns) { return (ns * (int)sizeof(float4) + 127) / 128 * 8 + 2; }   // float4
+
+template <bool GRAD, bool YUK, typename Boxes>
+__global__ void __launch_bounds__(kLeafThreads)
+leaf_eval_f32_kernel(const float4 *__restrict__ pts, Boxes bx, const int *__restrict__ list, int nboxes, int nl,
+                     const uint32_t *__restrict__ keys, const float *__restrict__ grid, int ns,
+                     const float *__restrict__ dens, int ldd, float scale, double ox, double oy, double oz, double width,
+                     double radius, float *__restrict__ phi, float *__restrict__ grad, const double *__restrict__ shift,
+                     float kappa) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4 *surf = reinterpret_cast<float4 *>(smem_raw);   // [nl][stride]
+    __shared__ float cen[kEvalLeaves][3];
+    __shared__ int box[kEvalLeaves], beg[kEvalLeaves], len[kEvalLeaves];
+    const int k0 = blockIdx.x * nl, m = min(nl, nboxes - k0), stride = eval_stride(ns);
+    if (threadIdx.x < m) {
+        const int b = list ? list[k0 + threadIdx.x] : k0 + (int)threadIdx.x;
+        box[threadIdx.x] = b;
+        box_range(bx, b, beg[threadIdx.x], len[threadIdx.x]);
+        int ax, ay, az;
+        demorton3(keys[b], ax, ay, az);
+        cen[threadIdx.x][0] = (float)(ox + (ax + 0.5) * width);
+        cen[threadIdx.x][1] = (float)(oy + (ay + 0.5) * width);
+        cen[threadIdx.x][2] = (float)(oz + (az + 0.5) * width);
+    }
+    __syncthreads();
+    const float r32 = (float)radius;   // no FP64 arithmetic per surface point
+    constexpr int kU = 2;               // staging loads in flight per thread
+    for (int e0 = threadIdx.x; e0 < m * ns; e0 += kU * kLeafThreads) {
+        float g[kU][3], d[kU];
+        int at[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const unsigned e = min(e0 + u * kLeafThreads, m * ns - 1), k = e / (unsigned)ns, j = e - k * ns;
+            const int c = 3 * (int)j;
+            g[u][0] = fmaf(r32, grid[c], cen[k][0]);
+            g[u][1] = fmaf(r32, grid[c + 1], cen[k][1]);
+            g[u][2] = fmaf(r32, grid[c + 2], cen[k][2]);
+            d[u] = dens[(int64_t)box[k] * ldd + j];
+            at[u] = (int)(k * stride * 4 + 8 * (j >> 1) + (j & 1));
+        }
+        float *o = reinterpret_cast<float *>(surf);   // past the last element: the last one again
+#pragma unroll
+        for (int u = 0; u < kU; ++u) o[at[u]] = g[u][0], o[at[u] + 2] = g[u][1], o[at[u] + 4] = g[u][2], o[at[u] + 6] = d[u];
+    }
+    __syncthreads();
+    for (int t = threadIdx.x;; t += kLeafThreads) {
+        int i = t, k = 0;
+        while (k < m && i >= len[k]) i -= len[k++];
+        if (k >= m) break;
+        i += beg[k];
+        const float4 *pr = surf + k * stride;
+        const float4 x = pts[i];
+        const float2 nx = make_float2(-x.x, -x.x), ny = make_float2(-x.y, -x.y), nz = make_float2(-x.z, -x.z);
+        float2 pot = make_float2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
+        for (int e = 0; e < ns / 2; ++e) pair_step<1, false, YUK>(pr, e, &nx, &ny, &nz, &pot, &gx, &gy, &gz, kappa);
+        const float f = scale * inv4pi<float>();
+        if (phi) phi[i] = (pot.x + pot.y) * f + (shift ? (float)shift[box[k]] : 0.f);   // the leaf's constant part
+        if (GRAD) {
+            grad[3 * (int64_t)i] = (gx.x + gx.y) * f;
+            grad[3 * (int64_t)i + 1] = (gy.x + gy.y) * f;
+            grad[3 * (int64_t)i + 2] = (gz.x + gz.y) * f;
+        }
+    }
+}
+
+// Leaves a block: as many as fill its threads at `mean` points a leaf, within 40 KB of surfaces (five blocks
+// an SM) and two blocks an SM in all.
+inline int eval_leaves(int nboxes, int64_t mean, int ns) {
+    int nl = (int)std::max<int64_t>(1, std::min<int64_t>(kEvalLeaves, kLeafThreads / std::max<int64_t>(1, mean)));
+    nl = std::min(nl, std::max(1, 40 * 1024 / (eval_stride(ns) * (int)sizeof(float4))));
+    return std::min(nl, std::max(1, nboxes / (2 * 152)));
 }
 
 template <typename T>
@@ -900,20 +947,32 @@ cudaError_t launch_leaf_eval(const fmm_ctx *ctx, const T *grid, const T *dens, i
     const double width = ctx->side / (double)(1 << d);
     const double radius = 2.95 * 0.5 * width;
     using P = typename Vec4<T>::type;
-    size_t smem = sizeof(P) * ctx->npts * (std::is_same<T, float>::value ? 2 : 1);   // FP32: + the pair layout
     const bool yuk = ctx->opt.kernel == FMM_YUKAWA;
     const T kappa = (T)ctx->opt.kappa;
     const LeafBoxes bx{ctx->leaf_off, (int)std::max<int64_t>(ctx->n, ctx->n_pts_all)};
-    auto go = [&](auto kern, T *g) {
-        kern<<<ctx->nleaf, kLeafThreads, smem, s>>>((const P *)ctx->pts, bx, nullptr, ctx->lev[d].keys, grid,
-                                                    ctx->npts, dens, ldd, scale, ctx->origin[0], ctx->origin[1],
-                                                    ctx->origin[2], width, radius, phi, g, shift, kappa);
-    };
-    if (grad)
-        yuk ? go(leaf_eval_kernel<T, true, true, LeafBoxes>, grad) : go(leaf_eval_kernel<T, true, false, LeafBoxes>, grad);
-    else
-        yuk ? go(leaf_eval_kernel<T, false, true, LeafBoxes>, nullptr)
-            : go(leaf_eval_kernel<T, false, false, LeafBoxes>, nullptr);
+    if constexpr (std::is_same<T, float>::value) {
+        const int nl = eval_leaves(ctx->nleaf, ctx->n / ctx->nleaf, ctx->npts);
+        auto go = [&](auto kern, float *g) {
+            kern<<<(ctx->nleaf + nl - 1) / nl, kLeafThreads, nl * eval_stride(ctx->npts) * sizeof(float4), s>>>(
+                (const float4 *)ctx->pts, bx, nullptr, ctx->nleaf, nl, ctx->lev[d].keys, grid, ctx->npts, dens, ldd, scale,
+                ctx->origin[0], ctx->origin[1], ctx->origin[2], width, radius, phi, g, shift, kappa);
+        };
+        if (grad) yuk ? go(leaf_eval_f32_kernel<true, true, LeafBoxes>, grad) : go(leaf_eval_f32_kernel<true, false, LeafBoxes>, grad);
+        else
+            yuk ? go(leaf_eval_f32_kernel<false, true, LeafBoxes>, nullptr)
+                : go(leaf_eval_f32_kernel<false, false, LeafBoxes>, nullptr);
+    } else {
+        auto go = [&](auto kern, T *g) {
+            kern<<<ctx->nleaf, kLeafThreads, sizeof(P) * ctx->npts, s>>>(
+                (const P *)ctx->pts, bx, nullptr, ctx->lev[d].keys, grid, ctx->npts, dens, ldd, scale, ctx->origin[0],
+                ctx->origin[1], ctx->origin[2], width, radius, phi, g, shift, kappa);
+        };
+        if (grad)
+            yuk ? go(leaf_eval_kernel<T, true, true, LeafBoxes>, grad) : go(leaf_eval_kernel<T, true, false, LeafBoxes>, grad);
+        else
+            yuk ? go(leaf_eval_kernel<T, false, true, LeafBoxes>, nullptr)
+                : go(leaf_eval_kernel<T, false, false, LeafBoxes>, nullptr);
+    }
     count_launch();
     return cudaGetLastError();
 }
@@ -926,15 +985,24 @@ cudaError_t launch_leaf_eval_rows(const fmm_ctx *ctx, int level, const int *list
     const double width = ctx->side / (double)(1 << level);
     const double radius = 2.95 * 0.5 * width;
     using P = typename Vec4<T>::type;
-    size_t smem = sizeof(P) * ctx->npts * (std::is_same<T, float>::value ? 2 : 1);
     const RowBoxes bx{begin, count, (int)std::max<int64_t>(ctx->n, ctx->n_pts_all)};
-    auto go = [&](auto kern, T *g) {
-        kern<<<n, kLeafThreads, smem, s>>>((const P *)ctx->pts, bx, list, ctx->lev[level].keys, grid, ctx->npts, dens,
-                                           ldd, (T)1, ctx->origin[0], ctx->origin[1], ctx->origin[2], width, radius,
-                                           phi, g, nullptr, (T)0);
-    };
-    if (grad) go(leaf_eval_kernel<T, true, false, RowBoxes>, grad);
-    else go(leaf_eval_kernel<T, false, false, RowBoxes>, nullptr);
+    if constexpr (std::is_same<T, float>::value) {
+        const int nl = eval_leaves(n, kLeafThreads / 4, ctx->npts);   // the counts are on the device: four leaves a block
+        auto go = [&](auto kern, float *g) {
+            kern<<<(n + nl - 1) / nl, kLeafThreads, nl * eval_stride(ctx->npts) * sizeof(float4), s>>>(
+                (const float4 *)ctx->pts, bx, list, n, nl, ctx->lev[level].keys, grid, ctx->npts, dens, ldd, 1.f,
+                ctx->origin[0], ctx->origin[1], ctx->origin[2], width, radius, phi, g, nullptr, 0.f);
+        };
+        grad ? go(leaf_eval_f32_kernel<true, false, RowBoxes>, grad) : go(leaf_eval_f32_kernel<false, false, RowBoxes>, nullptr);
+    } else {
+        auto go = [&](auto kern, T *g) {
+            kern<<<n, kLeafThreads, sizeof(P) * ctx->npts, s>>>((const P *)ctx->pts, bx, list, ctx->lev[level].keys, grid,
+                                                                ctx->npts, dens, ldd, (T)1, ctx->origin[0], ctx->origin[1],
+                                                                ctx->origin[2], width, radius, phi, g, nullptr, (T)0);
+        };
+        if (grad) go(leaf_eval_kernel<T, true, false, RowBoxes>, grad);
+        else go(leaf_eval_kernel<T, false, false, RowBoxes>, nullptr);
+    }
     count_launch();
     return cudaGetLastError();
 }

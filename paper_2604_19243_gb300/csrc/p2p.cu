@@ -796,11 +796,12 @@ template <typename T>
 __global__ void scatter_kernel(const T *__restrict__ near_phi, const T *__restrict__ near_grad,
                                const T *__restrict__ far_phi, const T *__restrict__ far_grad,
                                const int *__restrict__ perm, T *__restrict__ phi,
-                               T *__restrict__ grad, int64_t n, int64_t n_out) {
+                               T *__restrict__ grad, int64_t n, int64_t n_out, int64_t lo, int64_t hi) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int o = perm[i];
     if (!dbg_ok(o >= 0 && o < n_out, kDbgScatter)) return;
+    if (o < lo || o >= hi) return;   // another window's
     if (phi) {
         T v = 0;
         if (near_phi) v += near_phi[i];
@@ -832,8 +833,19 @@ template <typename T>
 cudaError_t launch_scatter(const T *near_phi, const T *near_grad, const T *far_phi,
                            const T *far_grad, const int *perm, T *phi, T *grad, int64_t n,
                            cudaStream_t s, int64_t n_out) {
-    scatter_kernel<T><<<blocks_for(n, 256), 256, 0, s>>>(near_phi, near_grad, far_phi, far_grad,
-                                                         perm, phi, grad, n, n_out < 0 ? n : n_out); count_launch();
+    const int64_t no = n_out < 0 ? n : n_out;
+    // The outputs' order is random in the sorted order: their sectors fill only if they stay in L2 until the last
+    // of their points is written.  Outputs larger than half of L2 are written in windows of that size, reading
+    // the sums once for each: 8.39M points (128 MB) 440 us in one pass, 254 in two, 251 in three, 312 in six;
+    // 4.19M points 131 in one, 120 in two.
+    constexpr int64_t kWindow = (int64_t)64 << 20;
+    // (The points of one virtual rank are a part of the outputs: the windows are those of the points.)
+    const int64_t bytes = n * (int64_t)sizeof(T) * ((phi ? 1 : 0) + (grad ? 3 : 0));
+    const int64_t windows = std::max<int64_t>(1, (bytes + kWindow - 1) / kWindow), w = (no + windows - 1) / windows;
+    for (int64_t k = 0; k < windows; ++k) {
+        scatter_kernel<T><<<blocks_for(n, 256), 256, 0, s>>>(near_phi, near_grad, far_phi, far_grad, perm, phi, grad, n,
+                                                             no, k * w, (k + 1) * w); count_launch();
+    }
     return cudaGetLastError();
 }
 

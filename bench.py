@@ -669,11 +669,12 @@ def main():
         # level's transforms and products run after the event that closes the phase)
         nfft = 2 * w.p
         m2l_flops = 8.0 * vpairs_upper * nfft * nfft * (nfft // 2 + 1)
-    tensor = args.precision in ("bf16x3", "bf16x6", "tf32x3", "fp16x3")
+    # products on the tensor cores per contraction: FP16X3 and the other split modes three, BF16X6 six; FP32's
+    # stencil six (three FP16 planes) and FP64's 36 (digits), their compress in FP32/FP64 arithmetic
+    products = {"fp16x3": (3, 3), "bf16x3": (3, 3), "tf32x3": (3, 3), "bf16x6": (6, 6), "fp32": (0, 6), "fp64": (0, 36)}
+    tensor = args.m2l != "fft"
     if tensor:
-        # products per contraction: BF16x6 six, the other split modes three (FP16X3 runs every
-        # contraction, the compress included, on hi/lo FP16 planes)
-        m_compress = m_stencil = 6 if args.precision == "bf16x6" else 3
+        m_compress, m_stencil = products[args.precision]
         tc_flops = m_compress * compress_flops + m_stencil * stencil_flops
         base = float(peaks["bf16_tflops_sustained"]) * (0.5 if args.precision == "tf32x3" else 1.0)
         m2l = {"bound": "tensor", "achieved": tc_flops / (m2l_ms * 1e-3) / 1e12,
@@ -686,20 +687,21 @@ def main():
     else:
         m2l = {"bound": "alu", "achieved": m2l_flops / (m2l_ms * 1e-3) / 1e12,
                "peak": fp32_peak_tf if not fp64 else None, "unit": "TFLOP/s",
-               "peak_basis": "measured FP32 FMA throughput (SIMT contraction)"}
+               "peak_basis": "measured FP32 FMA throughput"}
     if args.m2l == "fft":
         m2l_kernel = ("M2L phase, FFT form: transforms (fft_fwd_kernel, fft_inv_kernel), products "
                       "(fft_hadamard_kernel) and the equivalent-density GEMMs of levels 2 to depth - 1")
     else:
         m2l_kernel = ("M2L phase: compress + stencil GEMMs of all levels ("
-                      + ("gemm_tc_plane_kernel / gemm_tc_kernel" if tensor else "gemm_simt_kernel") + ")")
+                      + {"fp16x3": "gemm_f16_kernel", "fp32": "gemm_simt_kernel, gemm_f16_kernel",
+                         "fp64": "gemm_simt_kernel, gemm_f64_kernel"}.get(args.precision, "gemm_tc_plane_kernel, gemm_tc_kernel") + ")")
     m2l.update({"kernel": m2l_kernel,
                 "ms": m2l_ms, "v_pairs": vpairs, "algorithmic_flops": m2l_flops,
                 "timing": "CUDA events on the far-field stream: end of the upward pass to the start "
                           "of the leaf level's downward step"})
     m2l["frac"] = (m2l["achieved"] / m2l["peak"]) if m2l["peak"] else None
     m2l["traffic"] = None   # several launches per phase; the level-7 stencil's own figure follows
-    m2l["traffic_level7_stencil"] = recorded_traffic("gemm_tc_kernel_stencil_level7", source_digest("gemm_tc.cu"))
+    m2l["traffic_level7_stencil"] = recorded_traffic("gemm_f16_kernel_stencil_level7", source_digest("gemm_f16.cu"))
     # upward and downward passes in achieved GB/s (algorithmic bytes: every row read once and
     # written once, the points and outputs of the leaf steps once)
     es = 8 if fp64 else 4

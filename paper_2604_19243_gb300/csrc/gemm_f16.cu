@@ -84,6 +84,9 @@ struct F16Dev {
     int nstages, stage_bytes;
     int tmem_cols;
     int groups;                 // gridDim.z: groups of transfer vectors
+    // Both segments' rows and operators are scaled per chunk.  (Whether one is says nothing of the other: a
+    // segment of one chunk has one scale a row in either form.)
+    int chunked;
     float *Y;                   // FP32 rows (of group z: Y + z * y_group), or null
     int ldy;
     long long y_group;
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         const bool second = g.mode == GM_PARENT2 && tid == 1;
         if (second) op = t.cls;
         st.op[pos] = (short)op;
-        if (p.s0.nxs == 1) st.ws[pos] = second ? p.s1.ws[op] : p.s0.ws[op];
+        if (!p.chunked) st.ws[pos] = second ? p.s1.ws[op] : p.s0.ws[op];
     }
     tc_fence_before();
     __syncthreads();
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         // Each is loaded a segment before it is used.
         int src = nact > 0 ? source_row(g, st, me, 0) : -1, src1 = nact > 1 ? source_row(g, st, me, 1) : -1;
         float xs = src >= 0 ? __ldg(seg_of(0).xs + (size_t)src * seg_of(0).nxs) : 0.f;
-        const bool chunked = p.s0.nxs > 1;   // a factor per chunk instead of per segment
+        const bool chunked = p.chunked;   // a factor per chunk instead of per segment
         int slot = 0;
         for (int i = 0; i < nact; ++i) {
             const F16Seg &S = seg_of(i);
@@ -435,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         for (int i = 0; i < kHalf / 2; ++i) acc[i] = make_float2(0.f, 0.f);
         auto val = [&](int n) { return g.alpha * (n & 1 ? acc[n / 2].y : acc[n / 2].x); };
         bool ok = true;
-        const bool chunked = p.s0.nxs > 1;
+        const bool chunked = p.chunked;
         int slot = 0, b = 0;
         uint32_t phase = 0;
         for (int i = 0; i < nact && ok; ++i) {
@@ -746,6 +749,7 @@ cudaError_t gemm_f16(const fmm_ctx *ctx, const GemmCall &c, const F16Mat &W, con
     if (cols > 512) return cudaErrorInvalidValue;
     p.tmem_cols = cols;
     p.groups = c.groups;
+    p.chunked = c.xp_chunk_scales;
     p.Y = (float *)c.Y, p.ldy = c.ldy, p.y_group = c.y_group;
     if (c.Yp) {
         if (W.nsplit != 1 || c.groups != 1 || !c.yp_scale) return cudaErrorInvalidValue;

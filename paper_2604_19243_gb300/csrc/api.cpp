@@ -218,7 +218,7 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         const size_t pesz = ctx->f64m2l ? kDigitBytes : ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
         ctx->utp_plane = (long long)((size_t)rows * kw * pesz + 256) / 256 * 256;
         bool okp = pool_alloc(&ctx->UtP, (size_t)ctx->utp_plane * np, s) == cudaSuccess;
-        const size_t nsc = ctx->f16 && o.wide ? (size_t)(std::max(nsp, kw) + 63) / 64 : 1;   // scales a row
+        const size_t nsc = ctx->f16 ? (size_t)(std::max(nsp, kw) + 63) / 64 : 1;   // scales a row
         if (ctx->f16 || ctx->f32m2l || ctx->f64m2l)
             okp = okp && pool_alloc((void **)&ctx->Uscale, (size_t)rows * nsc * sizeof(float) + 16, s) == cudaSuccess &&
                   pool_alloc(&ctx->StP, stp * es + 16, s) == cudaSuccess;

@@ -167,7 +167,7 @@ cudaError_t FarSteps<T>::up(int l, cudaStream_t s) {
     c.W0 = O(l).up[0], c.w_stride = (int64_t)nsp * nsp;
     c.Y = rows_at<T>(A, ctx, l, nsp), c.ldy = nsp;
     const bool fused = f16 && !O(l).wide;   // one CTA holds a row: it writes the planes too
-    c.xp_chunk_scales = O(l).wide;
+    c.xp_chunk_scales = true;
     if (f16) {
         c.Xp = upP(l + 1), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l + 1);
         if (fused) c.Yp = upP(l), c.yp_ld = nsp, c.yp_plane = ctx->upp_plane, c.yp_scale = upS(l);
@@ -187,19 +187,19 @@ cudaError_t FarSteps<T>::compress(int l, cudaStream_t s) {
     c.X0 = rows_at<T>(A, ctx, l, nsp), c.ldx0 = nsp, c.k0 = nsp, c.W0 = o.compress;
     c.Y = ctx->tensor ? nullptr : rows_at<T>(ctx->Ut, ctx, l, kw), c.ldy = kw;   // tensor modes: planes only
     const bool fused = f16 && !o.wide;
-    c.xp_chunk_scales = o.wide;
+    c.xp_chunk_scales = true;
     if (f16) {
         c.Xp = upP(l), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l);
         if (!fused) c.Y = rows_at<T>(ctx->Ut, ctx, l, kw);
     }
     if (ctx->tensor && (!f16 || fused)) {
         c.Yp = utP(l), c.yp_ld = kw, c.yp_plane = ctx->utp_plane;
-        c.yp_scale = utS(l);
+        c.yp_scale = utS(l), c.yp_chunk_scales = !o.one_scale;
     }
     FMM_CUDA_TRY(gemm<T>(ctx, c, OP_COMPRESS + (adjoint ? OP_COUNT : 0), s));
     if (f16 && !fused)
         FMM_CUDA_TRY(launch_rows_planes((const float *)c.Y, 0, 1, kw, nullptr, ctx->lev[l].n, o.kinp, nullptr, 0, utP(l),
-                                        ctx->utp_plane, kw, utS(l), scales(o.kinp), 2, s));
+                                        ctx->utp_plane, kw, utS(l), ut_scales(), 2, s));
     return cudaSuccess;
 }
 
@@ -207,7 +207,7 @@ template <typename T> unsigned char *FarSteps<T>::utP(int l) const {
     const int pesz = ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
     return (unsigned char *)ctx->UtP + base(l) * kw * pesz;
 }
-template <typename T> float *FarSteps<T>::utS(int l) const { return ctx->Uscale ? ctx->Uscale + base(l) * (f16 ? scales(O(d).kinp) : 1) : nullptr; }
+template <typename T> float *FarSteps<T>::utS(int l) const { return ctx->Uscale ? ctx->Uscale + base(l) * ut_scales() : nullptr; }
 
 // rows of level l that can be sources: its boxes and, in a virtual rank's context, its ghosts
 template <typename T> int64_t FarSteps<T>::source_rows(int l) const {
@@ -246,7 +246,7 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
     st.groups = stencil_groups(o, l);
     if (st.groups > 1) st.Y = (float *)ctx->StP + ctx->stp_base[l], st.y_group = (long long)ctx->lev[l].n * kw;
     const bool fused = f16 && st.groups == 1 && !o.wide;
-    st.xp_chunk_scales = f16 && o.wide;
+    st.xp_chunk_scales = f16 && !o.one_scale;
     if (fused) {
         st.Y = nullptr;
         st.Yp = ctP(l), st.yp_ld = kw, st.yp_plane = ctx->ctp_plane, st.yp_scale = ctS(l);
@@ -272,7 +272,7 @@ cudaError_t FarSteps<T>::down(int l, cudaStream_t s) {
     c.Y = rows_at<T>(B, ctx, l, nsp), c.ldy = nsp;
     const bool children = l < d;   // the leaves' rows have no children to read them as planes
     const bool fused = f16 && children && !O(l).wide;
-    c.xp_chunk_scales = O(l).wide;
+    c.xp_chunk_scales = true;
     if (f16) {
         c.Xp = ctP(l), c.xp_ld = kw, c.xp_plane = ctx->ctp_plane, c.xp_scale = ctS(l);
         if (l >= 3) c.Xp1 = dnP(l - 1), c.xp1_ld = nsp, c.xp1_plane = ctx->upp_plane, c.xp1_scale = dnS(l - 1);
@@ -405,6 +405,7 @@ template <typename T>
 cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
     const int ns = h.ns, nsp = round_up(ns, 16);
     o.ns = ns, o.nsp = nsp, o.cplx = h.npts != h.ns, o.wide = nsp > 160;
+    o.one_scale = round_up(std::max(h.kin, h.kout), 16) <= 160;
     o.kin = adjoint ? h.kout : h.kin;
     o.kout = adjoint ? h.kin : h.kout;
     o.kinp = round_up(o.kin, 16), o.koutp = round_up(o.kout, 16);
@@ -420,15 +421,15 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
     if (ctx->f16) {
         std::vector<double> downs;
         for (int c = 0; c < 8; ++c) downs.insert(downs.end(), down[c].begin(), down[c].end());
-        FMM_CUDA_TRY(f16_upload(ctx, ups.data(), 8, ns, ns, nsp, 2, o.wide, &o.f_up));
-        FMM_CUDA_TRY(f16_upload(ctx, downs.data(), 8, ns, ns, nsp, 2, o.wide, &o.f_down));
-        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_compress : h.compress).data(), 1, o.kin, ns, nsp, 2, o.wide, &o.f_compress));
-        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_decompress : h.decompress).data(), 1, ns, o.kout, o.koutp, 2, o.wide,
+        FMM_CUDA_TRY(f16_upload(ctx, ups.data(), 8, ns, ns, nsp, 2, true, &o.f_up));
+        FMM_CUDA_TRY(f16_upload(ctx, downs.data(), 8, ns, ns, nsp, 2, true, &o.f_down));
+        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_compress : h.compress).data(), 1, o.kin, ns, nsp, 2, true, &o.f_compress));
+        FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_decompress : h.decompress).data(), 1, ns, o.kout, o.koutp, 2, true,
                                 &o.f_decompress));
     }
     if (ctx->f16 || ctx->f32m2l)
         FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_stencil : h.stencil).data(), kNumTransfer, o.kout, o.kin, o.kinp,
-                                ctx->f16 ? 2 : 3, o.wide, &o.f_stencil));
+                                ctx->f16 ? 2 : 3, ctx->f16 && !o.one_scale, &o.f_stencil));
     if (!h.fft_n) {   // the compressed M2L (the FFT form has its own transforms, fft.cu)
         FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_compress : h.compress, o.kin, ns, o.kinp, nsp, 1, &o.compress));
         if (ctx->f64m2l)

@@ -41,7 +41,7 @@ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 // power of two: [nsplit][K chunk][plane][16-byte unit of K][ncta output columns][16 B].
 struct F16Mat {
     void *data = nullptr;
-    float *scale = nullptr;     // 1 / scale per operator, or (two planes, wide) per operator and chunk
+    float *scale = nullptr;     // 1 / scale per operator, or per operator and chunk
     int n_out = 0;              // output columns (rows of the operator), nsplit * ncta when padded
     int ncta = 0, nsplit = 0;   // output columns per CTA, CTAs across the columns
     int K = 0, chunk = 0;       // padded input columns, and per stage
@@ -63,7 +63,10 @@ struct OpSet {
     // host-side shapes
     int ns = 0, nsp = 0;        // surface size and its padding to 16
     bool cplx = false;          // real form of complex operators (ns = 2 x the surface points)
-    bool wide = false;          // box vectors of more than 160 entries: FP16 planes of two scaled per 64 columns
+    bool wide = false;          // box vectors of more than 160 entries: no CTA of gemm_f16.cu holds a whole row
+    // compressed vectors of at most 160 entries: FP16X3's stencil has one scale a row and operator, and one
+    // accumulator a transfer vector (every other FP16X3 operand has a scale per 64 columns)
+    bool one_scale = false;
     int kin = 0, kinp = 0;      // M2L compressed source rank (Vi^T: kin x ns)
     int kout = 0, koutp = 0;    // M2L compressed target rank (Uo: ns x kout)
     int rcl = 0, rclp = 0;      // leaf-closing rank
@@ -439,9 +442,9 @@ struct GemmCall {
     const void *Xp = nullptr; int xp_ld = 0; int xp_rows = 0; long long xp_plane = 0;
     void *Yp = nullptr; int yp_ld = 0; long long yp_plane = 0;
     // FP16 planes (gemm_f16): 1 / scale of every row of Xp / Yp (of Xp per 64 columns if
-    // xp_chunk_scales), and the parent rows of PARENT2
+    // xp_chunk_scales, of Yp if yp_chunk_scales), and the parent rows of PARENT2
     const float *xp_scale = nullptr; bool xp_chunk_scales = false;
-    float *yp_scale = nullptr;
+    float *yp_scale = nullptr; bool yp_chunk_scales = true;
     const void *Xp1 = nullptr; int xp1_ld = 0; long long xp1_plane = 0;
     const float *xp1_scale = nullptr;
     // gemm_f16: the transfer vectors cut into `groups`, group z's sums written to Y + z * y_group
@@ -454,9 +457,9 @@ cudaError_t gemm_tc(const fmm_ctx *ctx, const GemmCall &g, int op_id, cudaStream
 // the operators W (PARENT2: W for the box's own rows, W1 for its parent's)
 cudaError_t gemm_f16(const fmm_ctx *ctx, const GemmCall &c, const F16Mat &W, const F16Mat *W1, cudaStream_t s);
 // `count` FP64 operators (rows x cols, K the padded cols) packed on the device into `planes` planes
-// (wide: scaled per 64 columns, as their rows)
-cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, int planes, bool wide,
-                       F16Mat *out);
+// (scaled as a whole, or per chunk of K as their rows)
+cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, int planes,
+                       bool chunk_scales, F16Mat *out);
 // rows list[i] (or i) < nrows: sum of `groups` partial rows (x_group apart), to FP32 rows y and / or
 // to FP16 planes with nsc scales a row (one, or one per 64 columns)
 cudaError_t launch_rows_planes(const float *x, long long x_group, int groups, int ldx, const int *list, int64_t nrows,
@@ -512,7 +515,8 @@ struct FarSteps {
     float *dnS(int l) const;
     float *ctS(int l) const;
     float *utS(int l) const;
-    int scales(int cols) const { return O(d).wide ? (cols + 63) / 64 : 1; }   // of a row of FP16 planes (FP16X3)
+    int scales(int cols) const { return (cols + 63) / 64; }   // of a row of FP16 planes (FP16X3)
+    int ut_scales() const { return f16 && !O(d).one_scale ? scales(O(d).kinp) : 1; }   // of a row of UtP
 };
 
 }  // namespace fmm

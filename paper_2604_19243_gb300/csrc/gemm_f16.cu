@@ -3,14 +3,13 @@
 // Operands.  Rows and operators are scaled by powers of two (largest entry just below 2^14) and cut
 // into FP16 terms of 11 bits each: two planes (hi, lo: 22 bits; FMM_FP16X3, products lo*hi, hi*lo,
 // hi*hi) or three (hi, mid, lo: 33 bits, which holds an FP32 value exactly unless it is more than 2^14
-// below the row's largest; FMM_FP32's M2L, the six products of order below three).  A row has one
-// scale, which loses at most 2^-39 of its largest entry; wide rows of two planes (OpSet::wide) one per
-// 64 columns.  The products add up in FP32 in tensor memory, smallest products first; since the
+// below the row's largest; FMM_FP32's M2L, the six products of order below three).  Rows and operators of
+// two planes have a scale per 64 columns, those of three planes, and of the stencil where the compressed
+// vectors fit one CTA, one for the whole row or operator.  The products add up in FP32 in tensor memory, smallest products first; since the
 // tensor core truncates when it adds, an accumulator takes one chunk's MMAs (at most four of them the
 // large products) before it is multiplied by its scales and added, correctly rounded, into FP32
-// registers.  Errors of the potentials against the direct sum in 64 bits, p = 6 (before: two-plane
-// sums drained once per transfer vector; FP32 in SIMT arithmetic): 60,001 points on the sphere, depth
-// 4, fp16x3 9.7e-7 (1.3e-6), fp32 5.1e-7 (7.1e-7).
+// registers.  The stencil of two planes is the exception where the compressed vectors fit one CTA (and
+// so have one scale a row): all chunks of a transfer vector add up in one accumulator.
 //
 // Layout.  One CTA computes a 128-row tile for ncta <= 160 output columns; blockIdx.y splits wider
 // outputs, blockIdx.z cuts the 189 transfer vectors of a stencil into groups whose partial sums go
@@ -87,13 +86,15 @@ struct F16Dev {
     // Both segments' rows and operators are scaled per chunk.  (Whether one is says nothing of the other: a
     // segment of one chunk has one scale a row in either form.)
     int chunked;
+    int seg_acc;                // a segment's chunks add up in one accumulator (one scale a row and operator)
     float *Y;                   // FP32 rows (of group z: Y + z * y_group), or null
     int ldy;
     long long y_group;
     unsigned char *yp;          // FP16 planes of the rows (nsplit == 1, groups == 1), or null
     long long yplane;
     int ldyp;
-    float *ys;                  // 1 / scale of every row of yp
+    float *ys;                  // 1 / scale of every row of yp, or per row and 64 columns: nys values a row
+    int nys;
     int *err;
     unsigned long long wait_ns;
 };
@@ -183,7 +184,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
     __shared__ SegTable st;
     __shared__ uint32_t mask[6];
     __shared__ int abort_flag, started_items;
-    __shared__ uint32_t pmax[2][kRows];
 
     const GemmDev &g = p.g;
     // the warp's number in a form that the compiler knows to be the same in all lanes
@@ -360,8 +360,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         // so that one warp's barrier waits (about 120 cycles each even if the phase is complete) run
         // beside the other's products.  A chunk's waits begin only when the other warp's for the chunk
         // before are over (turn_bar): the two use the stages and accumulators in turn, and a barrier's parity
-        // tells a phase from the one before only once that one is known to be complete.  The whole warp runs the loop, in uniform control flow and with
-        // the products unrolled, and one elected lane issues (mma_f16_elected).
+        // tells a phase from the one before only once that one is known to be complete.  A segment with one
+        // accumulator is one turn: its products are issued by one thread, in their order.  The whole warp runs
+        // the loop, in uniform control flow and with the products unrolled, and one elected lane issues
+        // (mma_f16_elected).
         const int mine = warp - kIssuer;
         int item = 0;
         const uint32_t elected = elect_one(), idesc = make_idesc(ncta, 0);
@@ -375,20 +377,24 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
             const bool second = g.mode == GM_PARENT2 && i == 1;
             const int K = second ? p.s1.K : p.s0.K, chunk = second ? p.s1.chunk : p.s0.chunk;
             for (int k0 = 0; k0 < K; k0 += chunk, ++item) {
-                if ((item & 1) != mine) {   // the other warp's
+                const bool first = !p.seg_acc || k0 == 0, last = !p.seg_acc || k0 + chunk >= K;   // of its accumulator
+                if (((p.seg_acc ? i : item) & 1) != mine) {   // the other warp's
                     if (++stage == p.nstages) stage = 0, phase ^= 1u;
-                    if (++b == kAcc) b = 0, aphase ^= 1u;
+                    if (last && ++b == kAcc) b = 0, aphase ^= 1u;
                     continue;
                 }
-                const bool ready = mbar_wait(&turn_bar[mine], turn, p.wait_ns) &&
+                const bool ready = (!first || mbar_wait(&turn_bar[mine], turn, p.wait_ns)) &&
                                    mbar_wait(&full_bar[stage], phase, p.wait_ns) &&
-                                   mbar_wait(&tempty_bar[b], aphase, p.wait_ns) && !*(volatile int *)&abort_flag;
+                                   (!first || mbar_wait(&tempty_bar[b], aphase, p.wait_ns)) &&
+                                   !*(volatile int *)&abort_flag;
                 if (!__all_sync(0xffffffffu, ready)) {
                     ok = false;
                     break;
                 }
-                if (elected) mbar_arrive(&turn_bar[mine ^ 1]);
-                turn ^= 1u;
+                if (last) {
+                    if (elected) mbar_arrive(&turn_bar[mine ^ 1]);
+                    turn ^= 1u;
+                }
                 tc_fence_after();
                 fence_proxy_async();   // the cp.async writes (generic proxy) -> tcgen05.mma
                 const int kv = min(chunk, K - k0), ksteps = kv >> 4;
@@ -405,16 +411,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
                     for (int k = 0; k < kSteps; ++k)   // a K step of 16: two units
                         if (k < ksteps)
                             mma_f16_elected(dt, ad + (uint64_t)(pa * ap + k * 2),
-                                            bd + (uint64_t)(pb * bp + (uint32_t)(k * 2 * ncta)), idesc, pr || k ? 1u : 0u,
+                                            bd + (uint64_t)(pb * bp + (uint32_t)(k * 2 * ncta)), idesc, pr || k || !first ? 1u : 0u,
                                             elected);
                 }
                 if (elected) {
                     mma_commit(&empty_bar[stage]);
-                    mma_commit(&tfull_bar[b]);
+                    if (last) mma_commit(&tfull_bar[b]);
                 }
                 __syncwarp();
                 if (++stage == p.nstages) stage = 0, phase ^= 1u;
-                if (++b == kAcc) b = 0, aphase ^= 1u;
+                if (last && ++b == kAcc) b = 0, aphase ^= 1u;
             }
         }
         if (elected) {
@@ -444,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         for (int i = 0; i < nact && ok; ++i) {
             const F16Seg &S = seg_of(i);
             const float *ws = S.ws + st.op[i] * S.nch;
-            for (int c = 0; c < S.nch; ++c) {
+            for (int c = 0; c < (p.seg_acc ? 1 : S.nch); ++c) {
                 const float w = chunked ? __ldg(ws + c) : 1.f;
                 if (!mbar_wait_warp(&tfull_bar[b], phase, p.wait_ns)) {
                     ok = false;
@@ -492,28 +498,44 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
                     *reinterpret_cast<float4 *>(y + n) =
                         make_float4(val(n), val(n + 1), val(n + 2), val(n + 3));
         }
-        if (p.yp) {   // the row's planes: every drain warp passes the barrier, also after a failed wait
-            uint32_t m = 0u;
+        if (p.yp) {   // the row's planes: every drain warp passes the barriers, also after a failed wait
+            // Largest entries of the row, per 64 columns, which can straddle the halves.  (They use the factors'
+            // memory, since another 3 KB would cost a stage: the first barrier follows every read of a factor.)
+            float(*const mx)[3][kRows] = reinterpret_cast<float(*)[3][kRows]>(&fac[0][0]);
+            uint32_t m[3] = {0u, 0u, 0u};
 #pragma unroll
             for (int n = 0; n < kHalf; ++n)
-                if (n < nc) m = max(m, __float_as_uint(fabsf(val(n))));
-            pmax[hf][row] = m;
-            __syncwarp();
+                if (n < nc) {
+                    const uint32_t v = __float_as_uint(fabsf(val(n)));
+                    const int ch = p.nys == 1 ? 0 : (c0 + n) >> 6;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) m[k] = max(m[k], ch == k ? v : 0u);
+                }
             asm volatile("bar.sync 2, 256;" ::: "memory");
-            float scale, inv;
-            row_scale(max(pmax[0][row], pmax[1][row]), scale, inv);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) mx[hf][k][row] = __uint_as_float(m[k]);
+            asm volatile("bar.sync 2, 256;" ::: "memory");
+            float scale[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                float inv;
+                row_scale(max(__float_as_uint(mx[0][k][row]), __float_as_uint(mx[1][k][row])), scale[k], inv);
+                // written by the thread that holds the first of the columns
+                if (ok && bx >= 0 && k < p.nys && k * 64 >= c0 && k * 64 < c0 + nc) p.ys[(size_t)bx * p.nys + k] = inv;
+            }
             if (ok && bx >= 0) {
-                if (hf == 0) p.ys[bx] = inv;
                 unsigned char *yp = p.yp + ((size_t)bx * p.ldyp + c0) * 2;
 #pragma unroll
                 for (int n = 0; n < kHalf; n += 8) {
                     if (n < nc && c0 + n < g.n_out) {
+                        const int ch = p.nys == 1 ? 0 : (c0 + n) >> 6;   // 8 columns lie within one
+                        const float sc = ch == 0 ? scale[0] : ch == 1 ? scale[1] : scale[2];
                         uint32_t w[NPL][4];
 #pragma unroll
                         for (int e = 0; e < 8; e += 2) {
                             uint32_t ha[NPL], hb[NPL];
-                            split_f16<NPL>(val(n + e) * scale, ha);
-                            split_f16<NPL>(val(n + e + 1) * scale, hb);
+                            split_f16<NPL>(val(n + e) * sc, ha);
+                            split_f16<NPL>(val(n + e + 1) * sc, hb);
 #pragma unroll
                             for (int k = 0; k < NPL; ++k) w[k][e / 2] = ha[k] | (hb[k] << 16);
                         }
@@ -587,16 +609,16 @@ rows_planes_kernel(const float *__restrict__ x, long long x_group, int groups, i
 
 // Operator k (block k): rows x cols FP64, row-major, into the stage form [nsplit][chunk][plane]
 // [unit][ncta rows][16 B] of the padded (nsplit * ncta) x K operator, and its 1 / scale: one for the
-// operator, or (wide) one per chunk.
+// operator, or (by_chunk) one per chunk.
 template <int NPL>
 __global__ void __launch_bounds__(256)
-pack_kernel(const double *__restrict__ w, int rows, int cols, int ncta, int nsplit, int K, int chunk, int wide,
-            unsigned char *__restrict__ out, float *__restrict__ inv_scale) {
+pack_kernel(const double *__restrict__ w, int rows, int cols, int ncta, int nsplit, int K, int chunk,
+            int by_chunk, unsigned char *__restrict__ out, float *__restrict__ inv_scale) {
     __shared__ double red[256], scale[kMaxChunks];
     const double *a = w + (size_t)blockIdx.x * rows * cols;
     const int nch = (K + chunk - 1) / chunk;
     for (int c = 0; c < nch; ++c) {
-        const int k0 = wide ? c * chunk : 0, kn = wide ? min(chunk, cols - k0) : cols;
+        const int k0 = by_chunk ? c * chunk : 0, kn = by_chunk ? min(chunk, cols - k0) : cols;
         double m = 0;
         for (int i = threadIdx.x; i < rows * kn; i += 256) m = fmax(m, fabs(a[(size_t)(i / kn) * cols + k0 + i % kn]));
         red[threadIdx.x] = m;
@@ -609,8 +631,8 @@ pack_kernel(const double *__restrict__ w, int rows, int cols, int ncta, int nspl
             int ex = 0;
             frexp(red[0], &ex);
             scale[c] = red[0] > 0 ? ldexp(1.0, 14 - ex) : 1.0;
-            if (wide || c == 0)
-                inv_scale[wide ? blockIdx.x * nch + c : blockIdx.x] = red[0] > 0 ? (float)ldexp(1.0, ex - 14) : 0.f;
+            if (by_chunk || c == 0)
+                inv_scale[by_chunk ? blockIdx.x * nch + c : blockIdx.x] = red[0] > 0 ? (float)ldexp(1.0, ex - 14) : 0.f;
         }
         __syncthreads();
     }
@@ -631,12 +653,10 @@ pack_kernel(const double *__restrict__ w, int rows, int cols, int ncta, int nspl
     }
 }
 
-// Two planes: 64 values of K a chunk (128-byte rows), evened out (48 + 48 + 48 for 144) unless the
-// rows are wide, which are scaled per 64 columns.
-int chunk_of(int K, int planes, bool wide) {
-    const int most = planes == 2 ? 64 : 32;
-    if (planes == 2 && wide) return most;
-    const int n = (K + most - 1) / most;
+// Two planes: 64 values of K a chunk, the columns of a scale.  Three: at most 32, evened out.
+int chunk_of(int K, int planes) {
+    if (planes == 2) return 64;
+    const int n = (K + 31) / 32;
     return round_up((K + n - 1) / n, 16);
 }
 
@@ -649,22 +669,21 @@ int chunk_of(int K, int planes, bool wide) {
 // many CTAs there are, and the number depends on the level alone: the same boxes give the same bits in
 // any partition.
 int stencil_groups(const OpSet &o, int level) {
-    // Real box vectors of more than 160 entries (p >= 7) in FP32 sums keep the sums of a box in one sequence: with
-    // charges of one sign, potentials in a deep tree are thousands of times their variation across a
-    // leaf, and another order of the same sums moves the gradients by as much as their own error (4e-5
-    // on 4.2M points at depth 6, p = 8).
-    if (o.wide && !o.cplx && !o.d_stencil.data) return 1;
+    // Real FP16X3 sums stay one sequence a box.  With charges of one sign a potential is 2^depth times its
+    // variation across a leaf, so that gradients carry the rounding of the sums (cube, p = 6: 2.3e-5 at depth 5,
+    // 4.7e-5 at depth 6, against FP64); another order of the same sums is no less exact, but gives gradients
+    // that differ by as much (2.2e-5 and 4.6e-5).  Sums of complex densities differ by 3e-6 at most (depth 5).
+    if (!o.cplx && !o.d_stencil.data && (o.f_stencil.planes == 2 || o.wide)) return 1;
     return level <= 3 ? 19 : level == 4 ? 9 : level == 5 ? 7 : 1;
 }
 
-cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, int planes, bool wide,
-                       F16Mat *out) {
-    const int chunk_scales = planes == 2 && wide;
+cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, int planes,
+                       bool chunk_scales, F16Mat *out) {
     out->n_out = rows, out->K = K, out->planes = planes;
     const int np = round_up(rows, 16);
     out->nsplit = (np + kMaxCols - 1) / kMaxCols;
     out->ncta = round_up((np + out->nsplit - 1) / out->nsplit, 16);
-    out->chunk = chunk_of(K, planes, wide);
+    out->chunk = chunk_of(K, planes);
     out->op_bytes = (size_t)out->nsplit * out->ncta * K * 2 * planes;
     void *d = nullptr, *ds = nullptr, *src = nullptr;
     FMM_CUDA_TRY(dev_malloc(&d, out->op_bytes * count));
@@ -750,10 +769,12 @@ cudaError_t gemm_f16(const fmm_ctx *ctx, const GemmCall &c, const F16Mat &W, con
     p.tmem_cols = cols;
     p.groups = c.groups;
     p.chunked = c.xp_chunk_scales;
+    p.seg_acc = c.mode == GM_STENCIL && npl == 2 && !c.xp_chunk_scales;
     p.Y = (float *)c.Y, p.ldy = c.ldy, p.y_group = c.y_group;
     if (c.Yp) {
         if (W.nsplit != 1 || c.groups != 1 || !c.yp_scale) return cudaErrorInvalidValue;
         p.yp = (unsigned char *)c.Yp, p.yplane = c.yp_plane, p.ldyp = c.yp_ld, p.ys = c.yp_scale;
+        p.nys = c.yp_chunk_scales ? (c.n_out + 63) / 64 : 1;
     }
     p.err = ctx->dev_flag;
     p.wait_ns = ctx->tc_wait_ns;

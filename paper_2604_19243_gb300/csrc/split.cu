@@ -568,7 +568,7 @@ fmm_status split_setup(fmm_ctx *ctx, int dg, int P) {
     const int es = ctx->fp64 ? 8 : 4;
     const bool f16 = ctx->f16;
     const OpSet &ops = ctx->fwd[d];
-    const int sc_s = ops.wide ? (nsp + 63) / 64 * 4 : 4, sc_k = ops.wide ? (ops.kinp + 63) / 64 * 4 : 4;   // bytes of a row's scales
+    const int sc_s = (nsp + 63) / 64 * 4, sc_k = ops.one_scale ? 4 : (ops.kinp + 63) / 64 * 4;   // bytes of a row's scales
     const int np = ctx->opt.precision == FMM_BF16X6 ? 3 : 2;
     const int pesz = ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
     std::vector<RowCopy> vex, gat, sca;

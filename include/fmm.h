@@ -56,17 +56,17 @@ typedef enum {
  * The near field (ULI), the S2U check potentials and D2T always run in FP32 SIMT arithmetic,
  * except under FMM_FP64 where everything is FP64. */
 typedef enum {
-    FMM_FP32 = 0,          /* FP32 SIMT, but for the dense VLI: FP32 values held as three FP16 terms
-                              (33 bits) on the tensor cores, FP32 sums; its error against 64 bits is
-                              no larger than FP32 arithmetic's */
+    FMM_FP32 = 0,          /* FP32 SIMT, but for the dense VLI of trees of depth <= 3 and of adaptive
+                              trees: FP32 values held as three FP16 terms (33 bits) on the tensor cores,
+                              FP32 sums; its error against 64 bits is no larger than FP32 arithmetic's */
     FMM_FP64 = 1,          /* FP64; inputs and outputs are double.  SIMT, but for the dense VLI: exact
                               products of 7-bit digits on the tensor cores (56 bits), FP64 sums */
     FMM_TF32X3 = 2,        /* contractions on tcgen05 tensor cores, 3 TF32 products (big/small split) */
     FMM_BF16X3 = 3,        /* contractions on tcgen05 tensor cores, 3 BF16 products (hi/lo split) */
     FMM_BF16X6 = 4,        /* contractions on tcgen05 tensor cores, 6 BF16 products (hi/mid/lo split) */
     FMM_FP16X3 = 5         /* contractions on tcgen05 tensor cores from FP16 hi/lo splits of power-of-two
-                              scaled operands (rows and operators scaled as a whole, or per 64 columns
-                              where a box vector has more than 160 entries), 3 FP16 products, about
+                              scaled operands (rows and operators scaled per 64 columns, or in the VLI
+                              as a whole where a compressed vector has at most 160 entries), 3 FP16 products, about
                               2^-22 relative per term, scales applied in FP32.  The leaf closing (the
                               pseudo-inverse of the downward check potentials) stays in FP32 SIMT, as
                               in every tensor-core mode.  No mean_free (FMM_EUNSUPPORTED). */

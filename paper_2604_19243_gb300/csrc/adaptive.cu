@@ -745,6 +745,7 @@ fmm_status adaptive_setup(fmm_ctx *ctx, int capacity) {
     A->capacity = capacity;
     A->rows = ctx->total_rows;
     cudaError_t e = build(ctx, A);
+    if (e == cudaSuccess && ctx->have_ops) e = upload_adaptive_planes(ctx);
     if (e != cudaSuccess) {
         const bool walk = e == cudaErrorInvalidValue;
         cudaGetLastError();

@@ -168,9 +168,10 @@ void free_ops(fmm_ctx *ctx) {
 // passes); the tiles of the VLI and the level sweeps are rebuilt for every tree.
 fmm_status ensure_workspace(fmm_ctx *ctx) {
     const int64_t need_rows = ctx->total_rows, need_nl = ctx->nleaf, need_n = ctx->n;
+    const bool f32p = f32_planes(ctx) || adaptive_planes(ctx);   // FP32 rows as planes
     // partial rows of the stencil's groups (gemm_f16.cu)
     size_t stp = 0;
-    if (ctx->f16 || ctx->f32m2l || ctx->f64m2l) {
+    if (ctx->f16 || f32p || ctx->f64m2l) {
         const OpSet &o = ctx->fwd[ctx->opt.depth];
         const int kw = std::max(std::max(o.kinp, o.koutp), 16);
         for (int l = 2; l <= ctx->opt.depth; ++l) {
@@ -178,7 +179,8 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
             if (stencil_groups(o, l) > 1) stp += (size_t)stencil_groups(o, l) * ctx->lev[l].n * kw;
         }
     }
-    if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n || stp > ctx->stp_vals))
+    if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n || stp > ctx->stp_vals ||
+                        (f32p && !ctx->UtP)))
         free_workspace(ctx);
     if (ctx->have_ws) {
         if (!ctx->tiles_ok) {
@@ -212,14 +214,15 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         {&ctx->near_grad, (size_t)n * 3 * vc * es}, {&ctx->far_phi, (size_t)n * vc * es},
         {&ctx->far_grad, (size_t)n * 3 * vc * es}, {&ctx->pts_qi, ctx->cplx ? (size_t)n * es : (size_t)16},
     };
-    if (ctx->tensor || ctx->f32m2l || ctx->f64m2l) {
-        const int np = ctx->f64m2l ? 1 : ctx->opt.precision == FMM_BF16X6 || ctx->f32m2l ? 3 : 2;
+    ctx->stp_vals = 0;
+    if (ctx->tensor || f32p || ctx->f64m2l) {
+        const int np = ctx->f64m2l ? 1 : ctx->opt.precision == FMM_BF16X6 || f32p ? 3 : 2;
         // (FP64: one array of digit rows)
         const size_t pesz = ctx->f64m2l ? kDigitBytes : ctx->opt.precision == FMM_TF32X3 ? 4 : 2;
         ctx->utp_plane = (long long)((size_t)rows * kw * pesz + 256) / 256 * 256;
         bool okp = pool_alloc(&ctx->UtP, (size_t)ctx->utp_plane * np, s) == cudaSuccess;
         const size_t nsc = ctx->f16 ? (size_t)(std::max(nsp, kw) + 63) / 64 : 1;   // scales a row
-        if (ctx->f16 || ctx->f32m2l || ctx->f64m2l)
+        if (ctx->f16 || f32p || ctx->f64m2l)
             okp = okp && pool_alloc((void **)&ctx->Uscale, (size_t)rows * nsc * sizeof(float) + 16, s) == cudaSuccess &&
                   pool_alloc(&ctx->StP, stp * es + 16, s) == cudaSuccess;
         if (ctx->f16) {
@@ -595,6 +598,10 @@ fmm_status fmm_precompute(fmm_ctx *ctx) {
         return fail(ctx, FMM_EUNSUPPORTED, "tensor-core contractions are not available in this library");
     }
     if (e != cudaSuccess) {
+        free_ops(ctx);
+        return cuda_fail(ctx, e, "operator upload");
+    }
+    if ((e = upload_adaptive_planes(ctx)) != cudaSuccess) {
         free_ops(ctx);
         return cuda_fail(ctx, e, "operator upload");
     }

@@ -76,7 +76,7 @@ template <typename T>
 cudaError_t gemm(const fmm_ctx *ctx, const GemmCall &c, int op_id, cudaStream_t s) {
     const int op = op_id % OP_COUNT;
     if (op == OP_CLOSE1 || op == OP_CLOSE2) return gemm_simt<T>(ctx, c, s);
-    if (ctx->f16 || (ctx->f32m2l && op == OP_STENCIL)) {
+    if (ctx->f16 || (f32_planes(ctx) && op == OP_STENCIL)) {
         const OpSet *set = op_id >= OP_COUNT ? ctx->adj : ctx->fwd;
         const OpSet &o = set[c.level];
         const F16Mat &w = op == OP_UP ? o.f_up : op == OP_COMPRESS ? o.f_compress
@@ -224,7 +224,8 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
     st.X0 = rows_at<T>(ctx->Ut, ctx, l, kw), st.ldx0 = kw, st.k0 = o.kinp;
     st.W0 = o.stencil, st.w_stride = (int64_t)o.koutp * o.kinp;
     st.Y = rows_at<T>(ctx->Ct, ctx, l, kw), st.ldy = kw;
-    if (ctx->tensor || ctx->f32m2l) {
+    const bool f32p = f32_planes(ctx);
+    if (ctx->tensor || f32p) {
         st.Xp = utP(l), st.xp_ld = kw, st.xp_rows = (int)ctx->lev[l].n, st.xp_plane = ctx->utp_plane;
         st.xp_scale = utS(l);
     }
@@ -237,8 +238,8 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
                                (unsigned char *)ctx->UtP + base(l) * kw * kDigitBytes, (int *)ctx->Uscale + base(l), nullptr,
                                ctx->lev[l].n, (double *)ctx->StP + ctx->stp_base[l], s);
         }
-    if (!f16 && !ctx->f32m2l) return gemm<T>(ctx, st, op, s);
-    if (ctx->f32m2l)   // FP32 rows (of the ghosts too) to three planes
+    if (!f16 && !f32p) return gemm<T>(ctx, st, op, s);
+    if (f32p)   // FP32 rows (of the ghosts too) to three planes
         FMM_CUDA_TRY(launch_rows_planes((const float *)st.X0, 0, 1, kw, nullptr, source_rows(l), o.kinp, nullptr, 0,
                                         utP(l), ctx->utp_plane, kw, utS(l), 1, 3, s));
     // FP32 mode reads FP32 rows next; FP16X3 planes, written by the stencil itself if one CTA holds
@@ -252,7 +253,7 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
         st.Yp = ctP(l), st.yp_ld = kw, st.yp_plane = ctx->ctp_plane, st.yp_scale = ctS(l);
     }
     FMM_CUDA_TRY(gemm<T>(ctx, st, op, s));
-    if (fused || (ctx->f32m2l && st.groups == 1)) return cudaSuccess;
+    if (fused || (f32p && st.groups == 1)) return cudaSuccess;
     return launch_rows_planes((const float *)st.Y, st.y_group, st.groups, kw, nullptr, ctx->lev[l].n, o.koutp,
                               f16 ? nullptr : (float *)rows_at<T>(ctx->Ct, ctx, l, kw), kw, f16 ? ctP(l) : nullptr,
                               ctx->ctp_plane, kw, f16 ? ctS(l) : nullptr, f16 ? scales(o.koutp) : 1, 2, s);
@@ -427,7 +428,7 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
         FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_decompress : h.decompress).data(), 1, ns, o.kout, o.koutp, 2, true,
                                 &o.f_decompress));
     }
-    if (ctx->f16 || ctx->f32m2l)
+    if (ctx->f16 || f32_planes(ctx))
         FMM_CUDA_TRY(f16_upload(ctx, (adjoint ? h.a_stencil : h.stencil).data(), kNumTransfer, o.kout, o.kin, o.kinp,
                                 ctx->f16 ? 2 : 3, ctx->f16 && !o.one_scale, &o.f_stencil));
     if (!h.fft_n) {   // the compressed M2L (the FFT form has its own transforms, fft.cu)
@@ -435,7 +436,7 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
         if (ctx->f64m2l)
             FMM_CUDA_TRY(f64_upload(ctx, (adjoint ? h.a_stencil : h.stencil).data(), kNumTransfer, o.kout, o.kin, o.kinp,
                                     &o.d_stencil));
-        else if (ctx->fp64)   // the others read planes
+        else if (ctx->fp64 || (ctx->f32m2l && !f32_planes(ctx)))   // the others read planes
             FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_stencil : h.stencil, o.kout, o.kin, o.koutp, o.kinp,
                                           kNumTransfer, &o.stencil));
         FMM_CUDA_TRY(upload_padded<T>(ctx, adjoint ? h.a_decompress : h.decompress, ns, o.kout, nsp, o.koutp, 1,
@@ -452,6 +453,16 @@ cudaError_t upload_set(fmm_ctx *ctx, const HostOps &h, bool adjoint, OpSet &o) {
 }
 
 }  // namespace
+
+cudaError_t upload_adaptive_planes(fmm_ctx *ctx) {
+    const int d = ctx->opt.depth;
+    if (!adaptive_planes(ctx) || ctx->fwd[d].f_stencil.data) return cudaSuccess;
+    const HostOps &h = *ctx->host_ops[d];   // Laplace: one set for every level
+    F16Mat m;
+    FMM_CUDA_TRY(f16_upload(ctx, h.stencil.data(), kNumTransfer, h.kout, h.kin, ctx->fwd[d].kinp, 3, false, &m));
+    for (OpSet &o : ctx->fwd) o.f_stencil = m;
+    return cudaSuccess;
+}
 
 cudaError_t upload_operators(fmm_ctx *ctx) {
     // the digit form of the FP64 stencil needs sums of K products to stay exact, in either direction

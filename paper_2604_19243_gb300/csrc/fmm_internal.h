@@ -158,7 +158,7 @@ struct fmm_ctx {
     bool cplx = false;          // complex densities and outputs (FMM_HELMHOLTZ)
     bool fft = false;           // M2L by FFT (FMM_M2L_FFT)
     bool f16 = false;           // FMM_FP16X3: contractions from two FP16 planes (gemm_f16.cu)
-    bool f32m2l = false;        // FMM_FP32: stencil from three FP16 planes (gemm_f16.cu)
+    bool f32m2l = false;        // FMM_FP32, dense M2L: f32_planes and the adaptive tree take the stencil from three FP16 planes
     bool f64m2l = false;        // FMM_FP64: stencil from integer digits (gemm_f64.cu; set by the operator upload)
     void *fft_ghat = nullptr;   // FFT M2L: the kernel's transforms [316][n n (n/2+1)] complex, storage type
     int *fft_surf = nullptr;    // FFT M2L: p^3 grid index of every surface point
@@ -450,6 +450,22 @@ struct GemmCall {
     // gemm_f16: the transfer vectors cut into `groups`, group z's sums written to Y + z * y_group
     int groups = 1; long long y_group = 0;
 };
+// FMM_FP32 on a uniform tree: the stencil from three FP16 planes (gemm_f16.cu) up to this depth, in SIMT
+// arithmetic below.  The planes' sums are the more exact (potentials of a cube of charges of one sign, depth 3,
+// p = 6: 2.7e-7 off FP64 against 6.6e-7), but gradients of such charges carry the rounding of the sums,
+// 2^depth times enlarged: 1.1e-5 in either form at depth 3, 2.4e-5 at depth 4, 5e-5 at depth 5, and the two
+// forms' gradients are 9.3e-6, 2.1e-5 and 4.3e-5 apart (the largest of p = 4, 6 and 8).  Up to depth 3 that is
+// within what a change of rounding may do.  (Clouds that need an adaptive tree have gradients of their
+// own size in the dense parts: 4e-6 apart at most, at depths 5 to 9.)
+constexpr int kF32PlaneDepth = 3;
+inline bool f32_planes(const fmm_ctx *ctx) { return ctx->f32m2l && ctx->opt.depth <= kF32PlaneDepth; }
+// FMM_FP32 with an adaptive tree set up: its stencil's planes (operators: upload_adaptive_planes, called by
+// whichever comes second of the set-up and the precomputation)
+inline bool adaptive_planes(const fmm_ctx *ctx) {
+    return ctx->f32m2l && ctx->adaptive && ctx->opt.kernel == FMM_LAPLACE;
+}
+cudaError_t upload_adaptive_planes(fmm_ctx *ctx);
+
 template <typename T>
 cudaError_t gemm_simt(const fmm_ctx *ctx, const GemmCall &g, cudaStream_t s);
 cudaError_t gemm_tc(const fmm_ctx *ctx, const GemmCall &g, int op_id, cudaStream_t s);

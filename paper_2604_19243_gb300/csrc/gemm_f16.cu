@@ -3,13 +3,13 @@
 // Operands.  Rows and operators are scaled by powers of two (largest entry just below 2^14) and cut
 // into FP16 terms of 11 bits each: two planes (hi, lo: 22 bits; FMM_FP16X3, products lo*hi, hi*lo,
 // hi*hi) or three (hi, mid, lo: 33 bits, which holds an FP32 value exactly unless it is more than 2^14
-// below the row's largest; FMM_FP32's M2L, the six products of order below three).  Rows and operators of
-// two planes have a scale per 64 columns, those of three planes, and of the stencil where the compressed
-// vectors fit one CTA, one for the whole row or operator.  The products add up in FP32 in tensor memory, smallest products first; since the
-// tensor core truncates when it adds, an accumulator takes one chunk's MMAs (at most four of them the
-// large products) before it is multiplied by its scales and added, correctly rounded, into FP32
-// registers.  The stencil of two planes is the exception where the compressed vectors fit one CTA (and
-// so have one scale a row): all chunks of a transfer vector add up in one accumulator.
+// below the row's largest; FMM_FP32's M2L in shallow and in adaptive trees, the six products of order
+// below three).  Rows and operators of two planes have a scale per 64 columns; those of three planes, and
+// the stencil's where the compressed vectors fit one CTA, one for the whole row or operator.  The products
+// add up in FP32 in tensor memory, smallest products first; since the tensor core truncates when it adds,
+// an accumulator takes one chunk's MMAs (at most four of them the large products) before it is multiplied
+// by its scales and added, correctly rounded, into FP32 registers.  Where the stencil of two planes has one
+// scale a row, all chunks of a transfer vector add up in one accumulator.
 //
 // Layout.  One CTA computes a 128-row tile for ncta <= 160 output columns; blockIdx.y splits wider
 // outputs, blockIdx.z cuts the 189 transfer vectors of a stencil into groups whose partial sums go
@@ -673,7 +673,7 @@ int stencil_groups(const OpSet &o, int level) {
     // variation across a leaf, so that gradients carry the rounding of the sums (cube, p = 6: 2.3e-5 at depth 5,
     // 4.7e-5 at depth 6, against FP64); another order of the same sums is no less exact, but gives gradients
     // that differ by as much (2.2e-5 and 4.6e-5).  Sums of complex densities differ by 3e-6 at most (depth 5).
-    if (!o.cplx && !o.d_stencil.data && (o.f_stencil.planes == 2 || o.wide)) return 1;
+    if (!o.cplx && o.f_stencil.planes == 2) return 1;
     return level <= 3 ? 19 : level == 4 ? 9 : level == 5 ? 7 : 1;
 }
 

@@ -1,5 +1,6 @@
 // SIMT (CUDA-core) form of the gathered GEMM of gemm_common.cuh, in FP32 or FP64: the FMM_FP32 and
-// FMM_FP64 contractions (but FP32's M2L, gemm_f16.cu) and the leaf closing of every mode.
+// FMM_FP64 contractions (but the M2L where gemm_f16.cu and gemm_f64.cu take it) and the leaf closing of
+// every mode.
 //
 // A CTA of 128 threads computes 64 rows x 64 columns (FP64: 32), 4 x 8 (4 x 4) a thread.  Rows and
 // operators go to shared memory as they lie in global memory (K contiguous), 64 bytes of K a stage, by

@@ -40,6 +40,26 @@ GRADIENTS = {
         -433.553925 296.304962 1650.71338 -164.558899 1914.01624 -383.136902
         916.584778 -1439.60339 379.218353 -1689.44019 733.041077 -457.328613
         """,
+    ("fp32", 6, 5, 20000): """
+        -271.47229 530.546082 1653.13391 -176.295609 -382.850311 -1074.22925
+        -150.85585 290.25943 1145.61865 -357.963623 -1428.53601 -946.206238
+        824.21991 582.674744 -997.928833 -456.460724 992.460754 -1208.0752
+        1053.38159 -766.326843 -670.746643 1883.73743 172.914658 -80.2765656
+        -132.252625 -305.791931 -1262.67126 -1268.31934 -958.301392 567.910828
+        -7.05098915 -1663.63635 -332.546478 -549.006958 280.18985 1231.08765
+        -430.354401 343.201233 1692.43127 -212.095383 1826.69275 -362.433411
+        976.777344 -1437.77954 361.888794 -1525.14697 779.133911 -364.748291
+        """,
+    ("fp32", 8, 4, 9001): """
+        -167.748932 224.343292 713.613098 684.383179 -129.419876 -172.992126
+        409.929077 224.38559 -548.593018 -421.16275 -111.402542 -592.931458
+        429.622284 -298.127533 -277.235107 -498.992432 145.139999 441.901184
+        223.674881 348.91452 -596.879089 57.9263535 378.565857 646.773071
+        404.501984 -385.007568 416.325836 249.265656 537.219543 -395.474182
+        -490.302032 -402.560028 -308.880615 534.984863 489.651123 159.238983
+        -132.681702 295.656586 -650.249512 41.9355888 267.110443 117.946396
+        -305.161987 -35.0608826 714.598755 -393.281006 -225.448853 470.173401
+        """,
 }
 
 

@@ -558,7 +558,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
 
 // Rows list[i] (i without a list), i < nrows: the sum of `groups` partial rows x + k * x_group in
 // order of k, written as FP32 (y, if not null) and as NPL planes (planes, if not null) with nsc
-// scales a row: one, or one per 64 columns.  One warp per row, at most 512 columns; bound by memory.
+// scales a row: one, or one per 64 columns.  One warp per row, 512 columns at a time (complex box vectors
+// have up to 976), which are read twice where a longer row has one scale; bound by memory.
 template <int NPL>
 __global__ void __launch_bounds__(256)
 rows_planes_kernel(const float *__restrict__ x, long long x_group, int groups, int ldx, const int *__restrict__ list,
@@ -569,41 +570,51 @@ rows_planes_kernel(const float *__restrict__ x, long long x_group, int groups, i
     const int r = list ? list[i] : i;
     const float *xr = x + (size_t)r * ldx;
     float4 v[4];
-    uint32_t m[4];
+    uint32_t m[4];   // largest entry of each v
+    auto load = [&](int c0) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = 4 * (lane + 32 * j);
-        m[j] = 0u;
-        v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < ncols) {
-            v[j] = *reinterpret_cast<const float4 *>(xr + c);
-            for (int k = 1; k < groups; ++k) {
-                const float4 a = *reinterpret_cast<const float4 *>(xr + k * x_group + c);
-                v[j].x += a.x, v[j].y += a.y, v[j].z += a.z, v[j].w += a.w;
+        for (int j = 0; j < 4; ++j) {
+            const int c = c0 + 4 * (lane + 32 * j);
+            m[j] = 0u;
+            v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c < ncols) {
+                v[j] = *reinterpret_cast<const float4 *>(xr + c);
+                for (int k = 1; k < groups; ++k) {
+                    const float4 a = *reinterpret_cast<const float4 *>(xr + k * x_group + c);
+                    v[j].x += a.x, v[j].y += a.y, v[j].z += a.z, v[j].w += a.w;
+                }
+                m[j] = max(max(__float_as_uint(fabsf(v[j].x)), __float_as_uint(fabsf(v[j].y))),
+                           max(__float_as_uint(fabsf(v[j].z)), __float_as_uint(fabsf(v[j].w))));
             }
-            if (y) *reinterpret_cast<float4 *>(y + (size_t)r * ldy + c) = v[j];
-            m[j] = max(max(__float_as_uint(fabsf(v[j].x)), __float_as_uint(fabsf(v[j].y))),
-                       max(__float_as_uint(fabsf(v[j].z)), __float_as_uint(fabsf(v[j].w))));
         }
-    }
-    if (!planes) return;
-    const uint32_t whole = __reduce_max_sync(0xffffffffu, max(max(m[0], m[1]), max(m[2], m[3])));
+    };
+    uint32_t whole = 0u;   // largest entry of the row
+    if (planes && nsc == 1)
+        for (int c0 = 0; c0 < ncols; c0 += 512) {
+            load(c0);
+            whole = max(whole, __reduce_max_sync(0xffffffffu, max(max(m[0], m[1]), max(m[2], m[3]))));
+        }
+    for (int c0 = 0; c0 < ncols; c0 += 512) {
+        if (!(planes && nsc == 1 && ncols <= 512)) load(c0);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = 4 * (lane + 32 * j);
-        float scale, inv;
-        // 64 columns: the lanes of one half of the warp
-        const uint32_t half = __reduce_max_sync(lane < 16 ? 0x0000ffffu : 0xffff0000u, m[j]);
-        row_scale(nsc == 1 ? whole : half, scale, inv);
-        if (c >= ncols) continue;
-        if (nsc == 1 ? j == 0 && lane == 0 : (lane & 15) == 0) inv_scale[(size_t)r * nsc + (nsc == 1 ? 0 : c / 64)] = inv;
-        uint32_t h[4][NPL];
-        split_f16<NPL>(v[j].x * scale, h[0]), split_f16<NPL>(v[j].y * scale, h[1]);
-        split_f16<NPL>(v[j].z * scale, h[2]), split_f16<NPL>(v[j].w * scale, h[3]);
+        for (int j = 0; j < 4; ++j) {
+            const int c = c0 + 4 * (lane + 32 * j);
+            if (y && c < ncols) *reinterpret_cast<float4 *>(y + (size_t)r * ldy + c) = v[j];
+            if (!planes) continue;
+            float scale, inv;
+            // 64 columns: the lanes of one half of the warp
+            const uint32_t half = __reduce_max_sync(lane < 16 ? 0x0000ffffu : 0xffff0000u, m[j]);
+            row_scale(nsc == 1 ? whole : half, scale, inv);
+            if (c >= ncols) continue;
+            if (nsc == 1 ? c == 0 : (lane & 15) == 0) inv_scale[(size_t)r * nsc + (nsc == 1 ? 0 : c / 64)] = inv;
+            uint32_t h[4][NPL];
+            split_f16<NPL>(v[j].x * scale, h[0]), split_f16<NPL>(v[j].y * scale, h[1]);
+            split_f16<NPL>(v[j].z * scale, h[2]), split_f16<NPL>(v[j].w * scale, h[3]);
 #pragma unroll
-        for (int k = 0; k < NPL; ++k)
-            *reinterpret_cast<uint2 *>(planes + k * plane_bytes + ((size_t)r * ldp + c) * 2) =
-                make_uint2(h[0][k] | (h[1][k] << 16), h[2][k] | (h[3][k] << 16));
+            for (int k = 0; k < NPL; ++k)
+                *reinterpret_cast<uint2 *>(planes + k * plane_bytes + ((size_t)r * ldp + c) * 2) =
+                    make_uint2(h[0][k] | (h[1][k] << 16), h[2][k] | (h[3][k] << 16));
+        }
     }
 }
 
@@ -715,7 +726,7 @@ cudaError_t launch_rows_planes(const float *x, long long x_group, int groups, in
                                float *inv_scale, int nsc, int nplanes, cudaStream_t s) {
     if (nrows <= 0) return cudaSuccess;
     if (nsc != 1 && nsc != (ncols + 63) / 64) return cudaErrorInvalidValue;
-    if (ncols > 512 || (ncols & 15)) return cudaErrorInvalidValue;
+    if (ncols & 15) return cudaErrorInvalidValue;
     auto go = [&](auto kern) {
         kern<<<(unsigned)((nrows + 7) / 8), 256, 0, s>>>(x, x_group, groups, ldx, list, (int)nrows, ncols, y, ldy,
                                                          (unsigned char *)planes, plane_bytes, ldp, inv_scale, nsc);

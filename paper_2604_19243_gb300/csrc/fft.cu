@@ -384,10 +384,10 @@ cudaError_t fft_vli(fmm_ctx *ctx, int l, const T *U, T *D, cudaStream_t s) {
     FMM_CUDA_TRY(gemm_simt<T>(ctx, c2, s));
     const V *ghat = (const V *)ctx->fft_ghat;
     const size_t fs = fwd_smem<T>(sh), is = inv_smem<T>(sh);
-    if (fs > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(fft_fwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs));
-    if (is > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(fft_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)is));
+    if (fs > 48 * 1024) FMM_CUDA_TRY(allow_all_shared(fft_fwd_kernel<T>));
+    if (is > 48 * 1024) FMM_CUDA_TRY(allow_all_shared(fft_inv_kernel<T>));
     const size_t hs = kHadSmem<T>;
-    FMM_CUDA_TRY(cudaFuncSetAttribute(fft_hadamard_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+    FMM_CUDA_TRY(allow_all_shared(fft_hadamard_kernel<T>));
     for (int ka0 = 0; ka0 < sh.n; ka0 += nka) {
         const int k = std::min(nka, sh.n - ka0);
         fft_fwd_kernel<T><<<(unsigned)nb, kFftThreads, fs, s>>>(sh, up.p, nsp, ctx->fft_surf, (int)nb, ka0, k, uh.p);

@@ -35,6 +35,21 @@ constexpr int kDigitBytes = 16;       // of one FP64 value as integer digits (ge
 constexpr int kNumTransfer = 316;     // [-3,3]^3 minus [-1,1]^3
 constexpr int kClassSlots = 189;      // transfer vectors with adjacent parents, per octant
 
+// Lets a kernel be launched with all of an SM's shared memory (227 KB, less its static part, which is also
+// returned).  The limit belongs to the function, for the whole process: set to the size of each launch, a
+// context on another thread could lower it between the setting and the launch, which is then refused.
+template <typename K>
+cudaError_t allow_all_shared(K kern, int *most = nullptr) {
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return e;
+    const int bytes = 227 * 1024 - (int)fa.sharedSizeBytes;
+    if (most) *most = bytes;
+    return fa.maxDynamicSharedSizeBytes == bytes
+               ? cudaSuccess
+               : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // Operators as FP16 planes for gemm_f16.cu (`count` of them, op_bytes apart), each scaled by one

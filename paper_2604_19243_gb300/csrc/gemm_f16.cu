@@ -769,10 +769,9 @@ cudaError_t gemm_f16(const fmm_ctx *ctx, const GemmCall &c, const F16Mat &W, con
     p.stage_bytes = round_up((kRows * (npl == 2 ? kRowBytes<2> : kRowBytes<3>) +
                               std::max(p.s0.chunk, p.s1.chunk) * W.ncta * 2) * npl, 1024);
     auto kern = npl == 2 ? gemm_f16_kernel<2> : gemm_f16_kernel<3>;
-    cudaFuncAttributes fa{};
-    FMM_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
-    const int budget = 227 * 1024 - 1024 - (int)fa.sharedSizeBytes;
-    p.nstages = std::min(kMaxStages, budget / p.stage_bytes);
+    int most = 0;
+    FMM_CUDA_TRY(allow_all_shared(kern, &most));
+    p.nstages = std::min(kMaxStages, (most - 1024) / p.stage_bytes);
     if (p.nstages < 2) return cudaErrorInvalidValue;
     int cols = 32;
     while (cols < kAcc * p.ncta) cols <<= 1;
@@ -790,7 +789,6 @@ cudaError_t gemm_f16(const fmm_ctx *ctx, const GemmCall &c, const F16Mat &W, con
     p.err = ctx->dev_flag;
     p.wait_ns = ctx->tc_wait_ns;
     const size_t smem = (size_t)p.nstages * p.stage_bytes + 1024;
-    FMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<dim3(ts.ntiles, W.nsplit, c.groups), kThreads, smem, s>>>(p);
     count_launch();
     return cudaGetLastError();

@@ -467,7 +467,7 @@ cudaError_t stencil_f64(const fmm_ctx *ctx, const GemmCall &c, const F64Mat &W, 
     p.ldy = c.ldy, p.y_group = c.y_group;
     p.err = ctx->dev_flag, p.wait_ns = ctx->tc_wait_ns;
     const size_t smem = (size_t)kStages * kStageBytes + 1024;
-    FMM_CUDA_TRY(cudaFuncSetAttribute(gemm_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FMM_CUDA_TRY(allow_all_shared(gemm_f64_kernel));
     gemm_f64_kernel<<<dim3(ts.ntiles, W.nsplit, c.groups), kThreads, smem, s>>>(p);
     count_launch();
     FMM_CUDA_TRY(cudaGetLastError());

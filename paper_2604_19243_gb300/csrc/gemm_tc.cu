@@ -853,10 +853,9 @@ cudaError_t gemm_tc(const fmm_ctx *ctx, const GemmCall &c, int op_id, cudaStream
     auto kern = plane ? (p.tf32 ? gemm_tc_plane_kernel<true> : gemm_tc_plane_kernel<false>)
                       : (p.tf32 ? gemm_tc_kernel<true> : gemm_tc_kernel<false>);
     const int threads = plane ? 384 : kTcThreads;
-    cudaFuncAttributes fa{};
-    FMM_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
-    const int budget = 227 * 1024 - 1024 - (int)fa.sharedSizeBytes;
-    p.nstages = std::min(plane ? kPlaneStages : 4, budget / stage_bytes);
+    int most = 0;
+    FMM_CUDA_TRY(allow_all_shared(kern, &most));
+    p.nstages = std::min(plane ? kPlaneStages : 4, (most - 1024) / stage_bytes);
     if (p.nstages < 2) return cudaErrorInvalidValue;
     // two accumulators of ncta columns; the drain reads 32 columns at a time, so the last read
     // of the second accumulator may extend 16 columns past it: keep that inside the allocation
@@ -882,7 +881,6 @@ cudaError_t gemm_tc(const fmm_ctx *ctx, const GemmCall &c, int op_id, cudaStream
         p.yp_ld = c.yp_ld;
     }
     const size_t smem = (size_t)p.nstages * stage_bytes + 1024;
-    FMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<dim3(ts.ntiles, (c.n_out + p.ncta - 1) / p.ncta), threads, smem, s>>>(p);
     count_launch();
     return cudaGetLastError();

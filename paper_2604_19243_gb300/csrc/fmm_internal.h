@@ -57,8 +57,7 @@ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 struct F16Mat {
     void *data = nullptr;
     float *scale = nullptr;     // 1 / scale per operator, or per operator and chunk
-    int n_out = 0;              // output columns (rows of the operator), nsplit * ncta when padded
-    int ncta = 0, nsplit = 0;   // output columns per CTA, CTAs across the columns
+    int ncta = 0, nsplit = 0;   // output columns per CTA, CTAs across the columns (the operator's rows, padded)
     int K = 0, chunk = 0;       // padded input columns, and per stage
     int planes = 0;             // 2: hi, lo (22 bits); 3: hi, mid, lo (33 bits)
     size_t op_bytes = 0;

@@ -43,7 +43,8 @@ namespace {
 
 constexpr int kRows = 128;
 constexpr int kMaxCols = 160;          // output columns per CTA
-constexpr int kProdWarps = 4, kProducers = 32 * kProdWarps, kWarpRows = kRows / kProdWarps;   // warps 0-3
+constexpr int kProdWarps = 4, kProducers = 32 * kProdWarps, kWarpRows = 32;   // warps 0-3, a row a thread
+static_assert(kProdWarps * kWarpRows == kRows);
 constexpr int kIssuer = 4;             // warps 4 and 5
 constexpr int kDrain0 = 6;             // warps 6-13
 constexpr int kLoader = 14;
@@ -176,8 +177,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
     extern __shared__ unsigned char smem_raw[];
     // full: a stage's A copies (one arrival a producer thread) and its operator copy (the loader's
     // expect_tx arrival); empty: the stage's MMAs done; tfull / tempty: an accumulator's MMAs done
-    // / drained; turn: an issuer may wait for its next chunk; fin: every MMA of an issuer done
+    // / drained; turn: an issuer may wait for its next chunk; fin: every MMA of an issuer done; fac: the
+    // row factors of a slot written (one arrival a producer warp; the full barriers' arrivals follow the
+    // asynchronous copies alone and make no ordinary store visible)
     __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tfull_bar[kAcc], tempty_bar[kAcc], turn_bar[2], fin_bar[2];
+    __shared__ uint64_t fac_bar[kFacRing];
     __shared__ uint32_t tmem_base;
     __shared__ int box[kRows];
     __shared__ float fac[kFacRing][kRows];
@@ -202,6 +206,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
             mbar_init(&tempty_bar[b], 8);
         }
         for (int k = 0; k < 2; ++k) mbar_init(&turn_bar[k], 1), mbar_init(&fin_bar[k], 1);
+        for (int k = 0; k < kFacRing; ++k) mbar_init(&fac_bar[k], kProdWarps);
         abort_flag = 0;
         started_items = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -246,11 +251,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
 
     if (warp < kProdWarps) {
         // ------------------------------------------------------------ producers
-        // Lane l looks up the source of its warp's row l mod 16, a segment ahead of the copies; the
-        // warp then copies its 16 rows, LPR lanes a row.
+        // Lane l looks up the source of its warp's row l, a segment ahead of the copies; the warp then
+        // copies its 32 rows, LPR lanes a row.
         constexpr int LPR = NPL == 2 ? 8 : 4, RPI = 32 / LPR, NP = kWarpRows / RPI;   // lanes a row, rows a pass, passes
         const int lr = lane / LPR, u = lane % LPR;               // its row of a pass and its unit
-        const int row = warp * kWarpRows + (lane & (kWarpRows - 1));
+        const int row = warp * kWarpRows + lane;
         const uint32_t sd = smem_u32(base) + a_offset<NPL>(warp * kWarpRows + lr, u);
         const RowPos me = row_pos(g, box[row]);
         int arrived = 0, stage = 0;
@@ -262,12 +267,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         float xs = src >= 0 ? __ldg(seg_of(0).xs + (size_t)src * seg_of(0).nxs) : 0.f;
         const bool chunked = p.chunked;   // a factor per chunk instead of per segment
         int slot = 0;
+        auto put_factor = [&](float f) {
+            fac[slot][row] = f;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&fac_bar[slot]);
+            slot = slot + 1 == kFacRing ? 0 : slot + 1;
+        };
         for (int i = 0; i < nact; ++i) {
             const F16Seg &S = seg_of(i);
-            if (!chunked) {
-                if (lane < kWarpRows) fac[slot][row] = xs * st.ws[i];
-                slot = slot + 1 == kFacRing ? 0 : slot + 1;
-            }
+            if (!chunked) put_factor(xs * st.ws[i]);
             const int src2 = i + 2 < nact ? source_row(g, st, me, i + 2) : -1;
             const float xs1 = src1 >= 0 ? __ldg(seg_of(i + 1).xs + (size_t)src1 * seg_of(i + 1).nxs) : 0.f;
             int off[NP];   // in 16-byte units from the first row; negative: no source
@@ -278,14 +286,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
             }
             ok = __all_sync(0xffffffffu, ok && !*(volatile int *)&abort_flag);
             for (int c = 0; c < S.nch && ok; ++c) {
+                if (chunked) {   // this chunk's factors; the next chunk's are loaded now
+                    put_factor(xs);
+                    if (c + 1 < S.nch) xs = src >= 0 ? __ldg(S.xs + (size_t)src * S.nxs + c + 1) : 0.f;
+                }
                 if (!mbar_wait_warp(&empty_bar[stage], phase, p.wait_ns)) {
                     ok = false;
                     break;
-                }
-                if (chunked) {   // this chunk's factors; the next chunk's are loaded now
-                    if (lane < kWarpRows) fac[slot][row] = xs;
-                    slot = slot + 1 == kFacRing ? 0 : slot + 1;
-                    if (c + 1 < S.nch) xs = src >= 0 ? __ldg(S.xs + (size_t)src * S.nxs + c + 1) : 0.f;
                 }
                 const int kv = min(S.chunk, S.K - c * S.chunk), units = kv >> 3;
                 if (u < units) {
@@ -446,18 +453,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
         bool ok = true;
         const bool chunked = p.chunked;
         int slot = 0, b = 0;
-        uint32_t phase = 0;
+        uint32_t phase = 0, fphase = 0;
+        // the row's factor in segment i (its chunk c), taken while the products of the one before run
+        auto factor = [&](int i, int c) {
+            const float w = chunked ? __ldg(seg_of(i).ws + st.op[i] * seg_of(i).nch + c) : 1.f;
+            ok = mbar_wait(&fac_bar[slot], fphase, p.wait_ns);
+            const float x = fac[slot][row];
+            if (++slot == kFacRing) slot = 0, fphase ^= 1u;
+            return chunked ? x * w : x;
+        };
+        float f = nact > 0 ? factor(0, 0) : 0.f;
         for (int i = 0; i < nact && ok; ++i) {
-            const F16Seg &S = seg_of(i);
-            const float *ws = S.ws + st.op[i] * S.nch;
-            for (int c = 0; c < (p.seg_acc ? 1 : S.nch); ++c) {
-                const float w = chunked ? __ldg(ws + c) : 1.f;
-                if (!mbar_wait_warp(&tfull_bar[b], phase, p.wait_ns)) {
-                    ok = false;
-                    break;
-                }
+            const int nd = p.seg_acc ? 1 : seg_of(i).nch;
+            for (int c = 0; c < nd; ++c) {
+                ok = __all_sync(0xffffffffu, ok && mbar_wait(&tfull_bar[b], phase, p.wait_ns));
+                if (!ok) break;
                 tc_fence_after();
-                const float f = chunked ? fac[slot][row] * w : fac[slot][row];
                 const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * ncta + c0);
 #pragma unroll
                 for (int n0 = 0; n0 < kHalf; n0 += 32) {
@@ -481,9 +492,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&tempty_bar[b]);
                 if (++b == kAcc) b = 0, phase ^= 1u;
-                if (chunked) slot = slot + 1 == kFacRing ? 0 : slot + 1;
+                if (c + 1 < nd) f = chunked ? factor(i, c + 1) : f;
+                else if (i + 1 < nact) f = factor(i + 1, 0);
             }
-            if (!chunked) slot = slot + 1 == kFacRing ? 0 : slot + 1;
+            ok = __all_sync(0xffffffffu, ok);
         }
         if (!ok) {
             atomicExch(p.err, FMM_ETIMEOUT);
@@ -690,7 +702,7 @@ int stencil_groups(const OpSet &o, int level) {
 
 cudaError_t f16_upload(fmm_ctx *ctx, const double *w, int count, int rows, int cols, int K, int planes,
                        bool chunk_scales, F16Mat *out) {
-    out->n_out = rows, out->K = K, out->planes = planes;
+    out->K = K, out->planes = planes;
     const int np = round_up(rows, 16);
     out->nsplit = (np + kMaxCols - 1) / kMaxCols;
     out->ncta = round_up((np + out->nsplit - 1) / out->nsplit, 16);

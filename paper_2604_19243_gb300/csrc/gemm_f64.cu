@@ -87,7 +87,8 @@ __device__ __forceinline__ int exponent_of(double m) {   // m < 2^e
 
 __global__ void __launch_bounds__(kThreads, 1) gemm_f64_kernel(const __grid_constant__ F64Dev p) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t full_bar[kStages], empty_bar[kStages], tfull_bar, tempty_bar, fin_bar;
+    // (as gemm_f16.cu's; ring: the row exponents of a slot written, one arrival a producer warp)
+    __shared__ uint64_t full_bar[kStages], empty_bar[kStages], tfull_bar, tempty_bar, fin_bar, ring_bar[kRing];
     __shared__ uint32_t tmem_base;
     __shared__ int box[kRows];
     __shared__ int ring[kRing][kRows];
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f64_kernel(const __grid_cons
             mbar_init(&empty_bar[s], 1);
         }
         mbar_init(&tfull_bar, 1), mbar_init(&tempty_bar, 8), mbar_init(&fin_bar, 1);
+        for (int k = 0; k < kRing; ++k) mbar_init(&ring_bar[k], kProducers / 32);
         abort_flag = started_items = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -157,6 +159,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f64_kernel(const __grid_cons
             const int next = i + 1 < nact ? source(i + 1) : -1;
             const int xe = src >= 0 ? __ldg(p.xe + src) : kNone, we = __ldg(p.we + seg[i].op);
             ring[slot][row] = xe == kNone || we == kNone ? kNone : xe == kBad || we == kBad ? kBad : xe + we;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ring_bar[slot]);
             slot = (slot + 1) % kRing;
             int from[8];
 #pragma unroll
@@ -280,9 +284,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f64_kernel(const __grid_cons
         for (int i = 0; i < kHalf; ++i) acc[i] = 0.0;
         bool ok = true;
         int slot = 0;
-        uint32_t phase = 0;
+        uint32_t phase = 0, rphase = 0;
         for (int i = 0; i < nact && ok; ++i) {
-            if (!mbar_wait_warp(&tfull_bar, phase, p.wait_ns)) {
+            if (!mbar_wait_warp(&tfull_bar, phase, p.wait_ns) || !mbar_wait_warp(&ring_bar[slot], rphase, p.wait_ns)) {
                 ok = false;
                 break;
             }
@@ -318,7 +322,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f64_kernel(const __grid_cons
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty_bar);
             phase ^= 1u;
-            slot = (slot + 1) % kRing;
+            if (++slot == kRing) slot = 0, rphase ^= 1u;
         }
         if (!ok) {
             atomicExch(p.err, FMM_ETIMEOUT);

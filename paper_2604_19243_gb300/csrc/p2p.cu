@@ -835,13 +835,16 @@ cudaError_t launch_scatter(const T *near_phi, const T *near_grad, const T *far_p
                            cudaStream_t s, int64_t n_out) {
     const int64_t no = n_out < 0 ? n : n_out;
     // The outputs' order is random in the sorted order: their sectors fill only if they stay in L2 until the last
-    // of their points is written.  Outputs larger than half of L2 are written in windows of that size, reading
-    // the sums once for each: 8.39M points (128 MB) 440 us in one pass, 254 in two, 251 in three, 312 in six;
-    // 4.19M points 131 in one, 120 in two.
-    constexpr int64_t kWindow = (int64_t)64 << 20;
+    // of their points is written.  Outputs larger than half of L2 are written in windows of that size, but in
+    // three at most: each reads the permutation and most of the sums again.  Potentials and gradients, in 1, 2, 3, 4
+    // and 8 windows: 8.39M points (128 MB) 462, 306, 317, 350, 550 us; 16.8M 1289, 949, 849, 858, 1138; 33.6M 2859,
+    // 2386, 2220, 2193, 2603; 67.1M 5938, 5330, 5245, 5203, 5925 (and 8342 in the 16 of 64 MB each); gradients
+    // or potentials alone likewise.  4.19M points (64 MB) take 94 us in one, 136 in two.
+    constexpr int64_t kWindow = (int64_t)64 << 20, kMostWindows = 3;
     // (The points of one virtual rank are a part of the outputs: the windows are those of the points.)
     const int64_t bytes = n * (int64_t)sizeof(T) * ((phi ? 1 : 0) + (grad ? 3 : 0));
-    const int64_t windows = std::max<int64_t>(1, (bytes + kWindow - 1) / kWindow), w = (no + windows - 1) / windows;
+    const int64_t windows = std::min(kMostWindows, std::max<int64_t>(1, (bytes + kWindow - 1) / kWindow));
+    const int64_t w = (no + windows - 1) / windows;
     for (int64_t k = 0; k < windows; ++k) {
         scatter_kernel<T><<<blocks_for(n, 256), 256, 0, s>>>(near_phi, near_grad, far_phi, far_grad, perm, phi, grad, n,
                                                              no, k * w, (k + 1) * w); count_launch();

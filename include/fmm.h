@@ -54,7 +54,12 @@ typedef enum {
 
 /* Arithmetic of the surface contractions (U2U, VLI, D2D and the check-to-equivalent steps).
  * The near field (ULI), the S2U check potentials and D2T always run in FP32 SIMT arithmetic,
- * except under FMM_FP64 where everything is FP64. */
+ * except under FMM_FP64 where everything is FP64.
+ * Beside its FP64 rows an FMM_FP64 context keeps 16 bytes per value of its compressed vectors and up to 19
+ * partial copies of the VLI sums of levels 2..5 (279 MB at a full level 5, p = 6); an FMM_FP32 context with
+ * an adaptive tree 6 bytes per value and such copies (half as large).  Where they do not fit into memory, the
+ * VLI runs in SIMT arithmetic from the rows alone.
+ * Densities that are not finite: no output that they reach is finite (infinite or NaN is unspecified). */
 typedef enum {
     FMM_FP32 = 0,          /* FP32 SIMT, but for the dense VLI of trees of depth <= 3 and of adaptive
                               trees: FP32 values held as three FP16 terms (33 bits) on the tensor cores,
@@ -66,8 +71,8 @@ typedef enum {
     FMM_BF16X6 = 4,        /* contractions on tcgen05 tensor cores, 6 BF16 products (hi/mid/lo split) */
     FMM_FP16X3 = 5         /* contractions on tcgen05 tensor cores from FP16 hi/lo splits of power-of-two
                               scaled operands (rows and operators scaled per 64 columns, or in the VLI
-                              as a whole where a compressed vector has at most 160 entries), 3 FP16 products, about
-                              2^-22 relative per term, scales applied in FP32.  The leaf closing (the
+                              as a whole where a compressed vector has at most 160 entries), 3 FP16
+                              products, about 2^-22 relative per term, scales applied in FP32.  The leaf closing (the
                               pseudo-inverse of the downward check potentials) stays in FP32 SIMT, as
                               in every tensor-core mode.  No mean_free (FMM_EUNSUPPORTED). */
 } fmm_precision;

@@ -919,13 +919,13 @@ static cudaError_t adaptive_stencil(fmm_ctx *ctx, GemmCall st, const AdaptiveLev
     const OpSet &o = ctx->fwd[l];
     const size_t rb = (size_t)ctx->lev[l].row_base;
     if constexpr (sizeof(T) == 8)
-        if (ctx->f64m2l) {
+        if (ctx->f64m2l && ctx->UtP) {
             st.groups = stencil_groups(o, l);
             st.y_group = (long long)ctx->lev[l].n * kw;
             return stencil_f64(ctx, st, o.d_stencil, L.kept, L.n_kept, (unsigned char *)ctx->UtP + rb * kw * kDigitBytes,
                                (int *)ctx->Uscale + rb, L.kept, L.n_kept, (double *)ctx->StP + ctx->stp_base[l], s);
         }
-    if (!ctx->f32m2l) return gemm_simt<T>(ctx, st, s);
+    if (!ctx->f32m2l || !ctx->UtP) return gemm_simt<T>(ctx, st, s);
     st.Xp = (unsigned char *)ctx->UtP + rb * kw * 2, st.xp_ld = kw, st.xp_plane = ctx->utp_plane;
     st.xp_scale = ctx->Uscale + rb;
     FMM_CUDA_TRY(launch_rows_planes((const float *)st.X0, 0, 1, kw, L.kept, L.n_kept, o.kinp, nullptr, 0, (void *)st.Xp,

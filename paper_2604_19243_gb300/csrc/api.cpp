@@ -126,7 +126,7 @@ void free_workspace(fmm_ctx *ctx) {
     for (int l = 0; l <= kMaxDepth; ++l)
         ctx->tiles_plain[l] = TileSet{}, ctx->tiles_cls[l] = TileSet{};
     free_async(ctx->tiles_all, s), free_async(ctx->masks_all, s);
-    ctx->have_ws = false;
+    ctx->have_ws = ctx->no_planes = false;
     ctx->ws_bytes = 0;
 }
 
@@ -180,7 +180,7 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         }
     }
     if (ctx->have_ws && (need_rows > ctx->ws_rows || need_nl > ctx->ws_nleaf || need_n > ctx->ws_n || stp > ctx->stp_vals ||
-                        (f32p && !ctx->UtP)))
+                        (f32p && !ctx->UtP && !ctx->no_planes)))
         free_workspace(ctx);
     if (ctx->have_ws) {
         if (!ctx->tiles_ok) {
@@ -198,14 +198,13 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
     ctx->ws_kw = kw;
     const int64_t rows = need_rows, nl = need_nl, n = need_n;
     const int vc = ctx->cplx ? 2 : 1;   // values per point (complex outputs)
-    // FP32 rows of the compressed vectors: the SIMT modes, and FP16X3 when no CTA holds a whole row
-    const size_t ut_bytes = !ctx->tensor || (ctx->f16 && o.wide) ? (size_t)rows * kw * es : (size_t)16;
+    // (tensor-core modes hand the compressed vectors over as split planes, UtP)
+    const size_t ut_bytes = !ctx->tensor ? (size_t)rows * kw * es : (size_t)16;
     struct A {
         void **p;
         size_t bytes;
     } allocs[] = {
         {&ctx->Uc, (size_t)rows * nsp * es},   {&ctx->Dc, (size_t)rows * nsp * es},
-        // tensor-core modes hand the compressed vectors over as split planes (UtP) instead
         {&ctx->Ut, ut_bytes},
         {&ctx->Ct, (size_t)rows * kw * es},
         {&ctx->Yc, (size_t)nl * o.rclp * es},
@@ -214,6 +213,16 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
         {&ctx->near_grad, (size_t)n * 3 * vc * es}, {&ctx->far_phi, (size_t)n * vc * es},
         {&ctx->far_grad, (size_t)n * 3 * vc * es}, {&ctx->pts_qi, ctx->cplx ? (size_t)n * es : (size_t)16},
     };
+    size_t total = 0;
+    for (auto &a : allocs) {
+        cudaError_t e = pool_alloc(a.p, std::max<size_t>(a.bytes, 16), s);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            free_workspace(ctx);
+            return fail(ctx, FMM_ENOMEM, "workspace allocation of " + std::to_string(a.bytes) + " bytes failed");
+        }
+        total += a.bytes;
+    }
     ctx->stp_vals = 0;
     if (ctx->tensor || f32p || ctx->f64m2l) {
         const int np = ctx->f64m2l ? 1 : ctx->opt.precision == FMM_BF16X6 || f32p ? 3 : 2;
@@ -238,22 +247,21 @@ fmm_status ensure_workspace(fmm_ctx *ctx) {
                   pool_alloc(&ctx->DnP, (size_t)ctx->upp_plane * 2, s) == cudaSuccess &&
                   pool_alloc(&ctx->CtP, (size_t)ctx->ctp_plane * 2, s) == cudaSuccess;
         }
+        ctx->stp_vals = stp;
+        // FP64, and FP32 with an adaptive tree, can do without: their M2L then runs in SIMT arithmetic
         if (!okp) {
             cudaGetLastError();
-            free_workspace(ctx);
-            return fail(ctx, FMM_ENOMEM, "workspace allocation failed (split planes)");
+            const bool spare = ctx->f64m2l || !(ctx->tensor || f32_planes(ctx));
+            if (spare) {
+                free_async(ctx->UtP, s), free_async(ctx->Uscale, s), free_async(ctx->StP, s);
+                ctx->no_planes = true;
+            }
+            if (!spare || upload_simt_stencils(ctx) != cudaSuccess) {
+                cudaGetLastError();
+                free_workspace(ctx);
+                return fail(ctx, FMM_ENOMEM, "workspace allocation failed (split planes)");
+            }
         }
-        ctx->stp_vals = stp;
-    }
-    size_t total = 0;
-    for (auto &a : allocs) {
-        cudaError_t e = pool_alloc(a.p, std::max<size_t>(a.bytes, 16), s);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            free_workspace(ctx);
-            return fail(ctx, FMM_ENOMEM, "workspace allocation of " + std::to_string(a.bytes) + " bytes failed");
-        }
-        total += a.bytes;
     }
     // rows that no step writes (levels 0-1, unused padding) must read as zero
     for (void **p : {&ctx->Uc, &ctx->Dc, &ctx->Ut, &ctx->Ct}) {
@@ -589,6 +597,7 @@ fmm_status fmm_precompute(fmm_ctx *ctx) {
     }
     try {
         e = upload_operators(ctx);
+        if (e == cudaSuccess) e = upload_adaptive_planes(ctx);
     } catch (const std::bad_alloc &) {
         free_ops(ctx);
         return fail(ctx, FMM_ENOMEM, "host memory exhausted in operator upload");
@@ -598,10 +607,6 @@ fmm_status fmm_precompute(fmm_ctx *ctx) {
         return fail(ctx, FMM_EUNSUPPORTED, "tensor-core contractions are not available in this library");
     }
     if (e != cudaSuccess) {
-        free_ops(ctx);
-        return cuda_fail(ctx, e, "operator upload");
-    }
-    if ((e = upload_adaptive_planes(ctx)) != cudaSuccess) {
         free_ops(ctx);
         return cuda_fail(ctx, e, "operator upload");
     }

@@ -14,6 +14,7 @@
 // at the points like D2T.  ULI is symmetric.
 #include <algorithm>
 #include <cmath>
+#include <new>
 #include <vector>
 
 #include "devutil.cuh"
@@ -190,7 +191,8 @@ cudaError_t FarSteps<T>::compress(int l, cudaStream_t s) {
     c.xp_chunk_scales = true;
     if (f16) {
         c.Xp = upP(l), c.xp_ld = nsp, c.xp_plane = ctx->upp_plane, c.xp_scale = upS(l);
-        if (!fused) c.Y = rows_at<T>(ctx->Ut, ctx, l, kw);
+        // (the stencil's output rows: it writes them once these have become planes)
+        if (!fused) c.Y = rows_at<T>(ctx->Ct, ctx, l, kw);
     }
     if (ctx->tensor && (!f16 || fused)) {
         c.Yp = utP(l), c.yp_ld = kw, c.yp_plane = ctx->utp_plane;
@@ -231,7 +233,7 @@ cudaError_t FarSteps<T>::stencil(int l, cudaStream_t s) {
     }
     const int op = OP_STENCIL + (adjoint ? OP_COUNT : 0);
     if constexpr (sizeof(T) == 8)
-        if (ctx->f64m2l) {   // (the ghosts' rows too)
+        if (ctx->f64m2l && ctx->UtP) {   // (the ghosts' rows too)
             st.groups = stencil_groups(o, l);
             st.y_group = (long long)ctx->lev[l].n * kw;
             return stencil_f64(ctx, st, o.d_stencil, nullptr, source_rows(l),
@@ -462,6 +464,24 @@ cudaError_t upload_adaptive_planes(fmm_ctx *ctx) {
     FMM_CUDA_TRY(f16_upload(ctx, h.stencil.data(), kNumTransfer, h.kout, h.kin, ctx->fwd[d].kinp, 3, false, &m));
     for (OpSet &o : ctx->fwd) o.f_stencil = m;
     return cudaSuccess;
+}
+
+cudaError_t upload_simt_stencils(fmm_ctx *ctx) try {
+    if (ctx->tensor || ctx->fft) return cudaSuccess;
+    for (OpSet *set : {ctx->fwd, ctx->adj})
+        for (int l = 0; l <= kMaxDepth; ++l) {
+            OpSet &o = set[l];
+            const HostOps &h = *ctx->host_ops[l];
+            for (int k = 0; k < l && !o.stencil; ++k)
+                if (ctx->host_ops[k] == ctx->host_ops[l]) o.stencil = set[k].stencil;
+            if (o.stencil) continue;
+            const std::vector<double> &w = set == ctx->adj ? h.a_stencil : h.stencil;
+            FMM_CUDA_TRY(ctx->fp64 ? upload_padded<double>(ctx, w, o.kout, o.kin, o.koutp, o.kinp, kNumTransfer, &o.stencil)
+                                   : upload_padded<float>(ctx, w, o.kout, o.kin, o.koutp, o.kinp, kNumTransfer, &o.stencil));
+        }
+    return cudaSuccess;
+} catch (const std::bad_alloc &) {
+    return cudaErrorMemoryAllocation;
 }
 
 cudaError_t upload_operators(fmm_ctx *ctx) {

@@ -244,6 +244,7 @@ struct fmm_ctx {
     void *near_phi = nullptr, *near_grad = nullptr;  // sorted-order outputs [n], [n x 3] (complex: x2)
     void *far_phi = nullptr, *far_grad = nullptr;
     size_t ws_bytes = 0;
+    bool no_planes = false;     // no memory for the planes (digits) of an M2L that has a SIMT form too
     int ws_kw = 0;
     void *grid_dev = nullptr;            // unit surface grid [ns x 3] in the storage type
     // host-pointer staging
@@ -479,6 +480,8 @@ inline bool adaptive_planes(const fmm_ctx *ctx) {
     return ctx->f32m2l && ctx->adaptive && ctx->opt.kernel == FMM_LAPLACE;
 }
 cudaError_t upload_adaptive_planes(fmm_ctx *ctx);
+// the SIMT form of the stencil operators that are there as digits or planes alone
+cudaError_t upload_simt_stencils(fmm_ctx *ctx);
 
 template <typename T>
 cudaError_t gemm_simt(const fmm_ctx *ctx, const GemmCall &g, cudaStream_t s);

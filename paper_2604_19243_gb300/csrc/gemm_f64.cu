@@ -1,7 +1,8 @@
 // FP64 M2L stencil on the FP16 tensor cores (tcgen05, sm_103a), exact products from integer digits.
 //
 // FP64 arithmetic runs at 1.25 TFLOP/s on this part, the FP16 tensor pipe at 2,000, so the stencil's
-// products are cut into integers that the tensor pipe multiplies and adds without rounding.  A row is
+// products are cut into integers that the tensor pipe multiplies and adds without rounding (the error-free
+// splitting of a matrix product into slices of Ozaki, Ogita, Oishi and Rump, 2012).  A row is
 // scaled by a power of two to at most 64 in size and written as eight digits of 7 bits, x = sum_i
 // d_i 2^(-7 i) with integers |d_i| <= 64 (56 bits below the row's largest entry; FP16 holds every
 // digit exactly), an operator likewise.  The products of digits i and j have the weight 2^(-7 (i + j));

@@ -180,6 +180,7 @@ void free_view(fmm_ctx *v, std::vector<void *> *owned) {
     free_workspace(v);
     if (owned)
         for (void *p : *owned) cudaFreeAsync(p, v->stream);
+    for (void *p : v->op_allocs) cudaFree(p);   // (its own alone: those of the context are shared)
     if (v->host_tiles) cudaFreeHost(v->host_tiles);
     if (v->tiles_ev) cudaEventDestroy(v->tiles_ev);
     delete v;

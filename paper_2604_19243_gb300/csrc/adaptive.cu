@@ -349,13 +349,17 @@ xli_kernel(const typename Pt4<T>::type *__restrict__ pts, const uint32_t *__rest
 // of shared memory and sums it at up to 64 points of the leaf, two a lane; leaves of up to 16 and 8
 // points have 2 and 4 groups of lanes share the surface.  (With one thread a point, leaves of some 30
 // points left three warps of four idle.)  A surface point is (c + r g) rounded once: in FP32 from the
-// centre and radius as sums of two FP32 numbers, since nine FP64 operations a point took longer than
+// centre and radius as sums of two FP32 numbers, the rounding errors of r g and of the sum carried along
+// (Dekker's and Knuth's error-free product and sum), since nine FP64 operations a point took longer than
 // the sums; a lane works out the centre of one box of 32 in FP64.
 // 1.05M points of an uneven cloud, p = 6: 2.73 -> 0.67 ms.
 constexpr int kWliWarps = kEvalThreads / 32, kWliChunk = 160;
 
 __device__ __forceinline__ float surface_point(float hi, float lo, float rhi, float rlo, float g) {
-    return hi + fmaf(rhi, g, fmaf(rlo, g, lo));
+    const float p = __fmul_rn(rhi, g), pe = __fmaf_rn(rhi, g, -p);   // r g = p + pe (+ rlo g)
+    const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);          // hi + p = s + e
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b));
+    return __fadd_rn(s, __fadd_rn(e, __fmaf_rn(rlo, g, __fadd_rn(lo, pe))));
 }
 __device__ __forceinline__ double surface_point(double hi, double, double rhi, double, double g) { return hi + rhi * g; }
 

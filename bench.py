@@ -670,9 +670,11 @@ def main():
         nfft = 2 * w.p
         m2l_flops = 8.0 * vpairs_upper * nfft * nfft * (nfft // 2 + 1)
     # products on the tensor cores per contraction: FP16X3 and the other split modes three, BF16X6 six; FP32's
-    # stencil six (three FP16 planes) and FP64's 36 (digits), their compress in FP32/FP64 arithmetic
+    # stencil six (three FP16 planes) up to depth 3 and none below, FP64's 36 (digits), their compress in
+    # FP32/FP64 arithmetic
     products = {"fp16x3": (3, 3), "bf16x3": (3, 3), "tf32x3": (3, 3), "bf16x6": (6, 6), "fp32": (0, 6), "fp64": (0, 36)}
-    tensor = args.m2l != "fft"
+    f32_simt = args.precision == "fp32" and w.depth > 3
+    tensor = args.m2l != "fft" and not f32_simt
     if tensor:
         m_compress, m_stencil = products[args.precision]
         tc_flops = m_compress * compress_flops + m_stencil * stencil_flops
@@ -693,7 +695,7 @@ def main():
                       "(fft_hadamard_kernel) and the equivalent-density GEMMs of levels 2 to depth - 1")
     else:
         m2l_kernel = ("M2L phase: compress + stencil GEMMs of all levels ("
-                      + {"fp16x3": "gemm_f16_kernel", "fp32": "gemm_simt_kernel, gemm_f16_kernel",
+                      + {"fp16x3": "gemm_f16_kernel", "fp32": "gemm_simt_kernel" + ("" if f32_simt else ", gemm_f16_kernel"),
                          "fp64": "gemm_simt_kernel, gemm_f64_kernel"}.get(args.precision, "gemm_tc_plane_kernel, gemm_tc_kernel") + ")")
     m2l.update({"kernel": m2l_kernel,
                 "ms": m2l_ms, "v_pairs": vpairs, "algorithmic_flops": m2l_flops,

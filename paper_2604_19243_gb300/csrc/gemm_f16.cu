@@ -26,9 +26,9 @@
 //
 // What bounds it: the tensor pipe on full tiles (eval on 4.2M cube points, p = 8: 0.6 us a chunk of 960
 // MMA cycles), the producers' instructions where most rows are absent (the sphere: 0.5 us a chunk of
-// 720).  M2L of all levels, far field alone, against the kernel with two 72 KB stages and products
-// issued by one lane: sphere 8.39M p = 6 2.7 -> 1.4 ms, cube 1M p = 6 1.7 -> 0.85 ms, cube 4.2M p = 8
-// 50 -> 13.5 ms; FP32 on cube 1M 13.8 (SIMT) -> 1.45 ms.
+// 720; there the tensor pipe is busy 54% of the time).  M2L of all levels, far field alone, against the
+// kernel with two 72 KB stages and products issued by one lane: sphere 8.39M p = 6 3.25 -> 1.63 ms, cube
+// 1M p = 6 1.89 -> 0.75 ms, cube 4.2M p = 8 53.6 -> 14.9 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -690,7 +690,9 @@ int chunk_of(int K, int planes) {
 // as long as one tile takes: levels 2 and 3 have at most 8 tiles (one a class), level 4 8 to 32 and
 // level 5 16 to 256.  The groups' partial rows are added in order, so a result does not depend on how
 // many CTAs there are, and the number depends on the level alone: the same boxes give the same bits in
-// any partition.
+// any partition.  Step of 20k points (FP32, depth 3), Helmholtz evaluation (131k, depth 4), FP64 (100k,
+// depth 4): 359, 809, 10083 us; half as many groups 358, 819, 10198; twice as many 359, 834, 10090; none
+// 506, 1063, 10342.
 int stencil_groups(const OpSet &o, int level) {
     // Real FP16X3 sums stay one sequence a box.  With charges of one sign a potential is 2^depth times its
     // variation across a leaf, so that gradients carry the rounding of the sums (cube, p = 6: 2.3e-5 at depth 5,

@@ -463,6 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f16_kernel(const __grid_cons
             return chunked ? x * w : x;
         };
         float f = nact > 0 ? factor(0, 0) : 0.f;
+        ok = __all_sync(0xffffffffu, ok);   // (a wait can run out in some lanes alone)
         for (int i = 0; i < nact && ok; ++i) {
             const int nd = p.seg_acc ? 1 : seg_of(i).nch;
             for (int c = 0; c < nd; ++c) {

@@ -698,7 +698,8 @@ int stencil_groups(const OpSet &o, int level) {
     // Real FP16X3 sums stay one sequence a box.  With charges of one sign a potential is 2^depth times its
     // variation across a leaf, so that gradients carry the rounding of the sums (cube, p = 6: 2.3e-5 at depth 5,
     // 4.7e-5 at depth 6, against FP64); another order of the same sums is no less exact, but gives gradients
-    // that differ by as much (2.2e-5 and 4.6e-5).  Sums of complex densities differ by 3e-6 at most (depth 5).
+    // that differ by as much (2.2e-5 and 4.6e-5).  Sums of complex densities differ by 3e-6 at most
+    // (depths 2 to 5).
     if (!o.cplx && o.f_stencil.planes == 2) return 1;
     return level <= 3 ? 19 : level == 4 ? 9 : level == 5 ? 7 : 1;
 }
